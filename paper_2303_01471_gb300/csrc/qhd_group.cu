@@ -76,7 +76,7 @@ __device__ __noinline__ void group_prep(const GroupArgs &a, const GroupClass &g,
     uint64_t kt_turns[3];
     double kt_fd[3];
     for (int64_t i = tid; i < (j_hi - j_lo) * pa.batch; i += nth)
-        prep_coefficients(pa, j_lo + i / pa.batch, i % pa.batch, kt_turns, kt_fd, true);
+        pa.pot[j_lo * pa.batch + i] = prep_coefficients(pa, j_lo + i / pa.batch, i % pa.batch, kt_turns, kt_fd);
     // kinetic rows (jl, b) of steps jl < cnt: CTA crank takes rows crank, crank + CL, ...
     __shared__ uint64_t s_k[3];
     __shared__ double s_fd[3];
@@ -84,9 +84,10 @@ __device__ __noinline__ void group_prep(const GroupArgs &a, const GroupClass &g,
     const int64_t rows = k_hi > j_lo ? (k_hi - j_lo) * pa.kt_batch : 0;
     for (int64_t r = crank; r < rows; r += GROUP_CL) {
         const int64_t jl = j_lo + r / pa.kt_batch, b = r % pa.kt_batch;
-        if (threadIdx.x == 0) prep_coefficients(pa, jl, b, s_k, s_fd, false);
+        if (threadIdx.x == 0) prep_coefficients(pa, jl, b, s_k, s_fd);
         __syncthreads();
-        for (int i = threadIdx.x; i < pa.ksum; i += PLANE_THREADS) prep_kinetic_entry(pa, jl, b, i, s_k, s_fd);
+        float4 *out = pa.kt + (jl * pa.kt_batch + b) * pa.ksum;
+        for (int i = threadIdx.x; i < pa.ksum; i += PLANE_THREADS) out[i] = prep_kinetic_entry(pa, i, s_k, s_fd);
         __syncthreads();
     }
     __threadfence();

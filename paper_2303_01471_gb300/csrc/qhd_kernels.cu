@@ -22,6 +22,7 @@
 // so the FP32 sine/cosine only ever sees a reduced argument.
 #include "qhd_device.cuh"
 #include "qhd_kernels.h"
+#include "qhd_launch.cuh"
 #include "qhd_sched.cuh"
 #include "qhd_prep.cuh"
 
@@ -51,8 +52,10 @@ __global__ void __launch_bounds__(ROW_THREADS) k_row(RowArgs a) {
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
     float2 *smem = reinterpret_cast<float2 *>(smem4 + PHASE_TAB);
+    grid_release();
     load_phase_tab(ptab, a.ptab);
     __syncthreads();
+    grid_wait();
     const int lpb = blockDim.x / T;
     const int line = threadIdx.x / T, t = threadIdx.x % T;
     const int64_t row = (int64_t)blockIdx.x * lpb + line;
@@ -95,6 +98,8 @@ __global__ void __launch_bounds__(W * LineCfg<N>::T, N <= 256 ? 4 : 1) k_axis(Ax
     const int64_t o = blockIdx.x / tiles;
     const int64_t ci = (blockIdx.x - o * tiles) * W + c;
     float2 *g = a.psi + o * (int64_t)N * a.inner + ci;
+    grid_release();
+    grid_wait();
     float2 x[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) x[e] = g[(int64_t)(t + T * e) * a.inner];
@@ -160,8 +165,10 @@ __global__ void __launch_bounds__(ROW_THREADS) k_oned(OneDArgs a) {
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
     float2 *smem = reinterpret_cast<float2 *>(smem4 + PHASE_TAB);
+    grid_release();
     load_phase_tab(ptab, a.ptab);
     __syncthreads();
+    grid_wait();
     const int lpb = blockDim.x / T;
     const int line = threadIdx.x / T, t = threadIdx.x % T;
     const int64_t row = (int64_t)blockIdx.x * lpb + line;
@@ -219,14 +226,27 @@ __global__ void k_prep(PrepArgs a) {
     const int64_t b = blockIdx.y;
     __shared__ uint64_t s_k[3];
     __shared__ double s_fd[3];
-    if (threadIdx.x == 0) prep_coefficients(a, jl, b, s_k, s_fd);
+    grid_release();
+    uint64_t pot = 0;
+    if (threadIdx.x == 0) pot = prep_coefficients(a, jl, b, s_k, s_fd);
     __syncthreads();
-    if (jl >= a.cnt || b >= a.kt_batch) return;
-    for (int i = threadIdx.x; i < a.ksum; i += blockDim.x) prep_kinetic_entry(a, jl, b, i, s_k, s_fd);
+    // the schedules and the potential's scale were loaded under a synchronisation,
+    // the tables are read by the passes before: compute first, wait, then write
+    const bool row = jl < a.cnt && b < a.kt_batch;
+    const bool one = row && (int)threadIdx.x < a.ksum;
+    const float4 first = one ? prep_kinetic_entry(a, threadIdx.x, s_k, s_fd) : make_float4(0.f, 0.f, 0.f, 0.f);
+    grid_wait();
+    if (threadIdx.x == 0) a.pot[jl * a.batch + b] = pot;
+    if (!one) return;
+    float4 *out = a.kt + (jl * a.kt_batch + b) * a.ksum;
+    out[threadIdx.x] = first;
+    for (int i = threadIdx.x + blockDim.x; i < a.ksum; i += blockDim.x) out[i] = prep_kinetic_entry(a, i, s_k, s_fd);
 }
 
 // ------------------------------------------------------------ small kernels
 __global__ void k_uniform(float2 *psi, int64_t count, float v) {
+    grid_release();
+    grid_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x)
         psi[i] = make_float2(v, 0.0f);
@@ -307,6 +327,8 @@ __global__ void k_obs_partial(ObsArgs a) {
     const float2 *psi = a.psi + b * a.g;
     const double *f = a.f64 + b * a.g;
     const InstDev &ip = a.inst[b];
+    grid_release();
+    grid_wait();
     double sn = 0.0, sf = 0.0, sp = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.g;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -342,6 +364,8 @@ __global__ void k_obs_partial(ObsArgs a) {
 __global__ void k_obs_final(ObsArgs a) {
     const int64_t b = blockIdx.x;
     __shared__ double sh[3][256];
+    grid_release();
+    grid_wait();
     for (int k = 0; k < 3; ++k) {
         double s = 0.0;
         for (int i = threadIdx.x; i < a.nblk; i += blockDim.x) s += a.partial[(b * a.nblk + i) * 3 + k];
@@ -365,8 +389,7 @@ static cudaError_t row_impl(const RowArgs &a, cudaStream_t s) {
     const int lpb = ROW_THREADS / C::T;
     const int64_t blocks = (a.rows + lpb - 1) / lpb;
     const size_t sm = PHASE_TAB * sizeof(float4) + (C::TWO_STAGE ? (size_t)lpb * S * sizeof(float2) : 0);
-    k_row<N><<<(unsigned)blocks, ROW_THREADS, sm, s>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(a.rows * N < OVERLAP_POINTS, k_row<N>, dim3((unsigned)blocks), dim3(ROW_THREADS), sm, s, a);
 }
 
 template <int N, int W>
@@ -376,8 +399,7 @@ static cudaError_t axis_w_impl(const AxisArgs &a, cudaStream_t s) {
     const int64_t blocks = a.planes * (a.inner / W);
     // exchange buffer, then the column partial sums of the zero-mode split
     const size_t xch = (C::TWO_STAGE ? (size_t)W * S * sizeof(float2) : 0) + (size_t)W * C::T * sizeof(float2);
-    k_axis<N, W><<<(unsigned)blocks, W * C::T, xch, s>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(a.planes * a.inner * N < OVERLAP_POINTS, k_axis<N, W>, dim3((unsigned)blocks), dim3(W * C::T), xch, s, a);
 }
 
 template <int N>
@@ -398,8 +420,7 @@ static cudaError_t oned_impl(const OneDArgs &a, cudaStream_t s) {
     const int lpb = ROW_THREADS / C::T;
     const int64_t blocks = (a.batch + lpb - 1) / lpb;
     const size_t sm = PHASE_TAB * sizeof(float4) + (C::TWO_STAGE ? (size_t)lpb * S * sizeof(float2) : 0);
-    k_oned<N><<<(unsigned)blocks, ROW_THREADS, sm, s>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(true, k_oned<N>, dim3((unsigned)blocks), dim3(ROW_THREADS), sm, s, a);
 }
 
 #define QHD_DISPATCH_N(n, fn, ...)                        \
@@ -423,15 +444,13 @@ cudaError_t launch_oned(int n, const OneDArgs &a, cudaStream_t s) { QHD_DISPATCH
 
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
     dim3 grid((unsigned)(a.cnt + 1), (unsigned)a.batch);
-    k_prep<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(true, k_prep, grid, dim3(256), 0, s, a);
 }
 
 cudaError_t launch_uniform(float2 *psi, int64_t count, float value, cudaStream_t s) {
     int64_t blocks = (count + 255) / 256;
     if (blocks > 152 * 32) blocks = 152 * 32;
-    k_uniform<<<(unsigned)blocks, 256, 0, s>>>(psi, count, value);
-    return cudaGetLastError();
+    return launch_overlapped(true, k_uniform, dim3((unsigned)blocks), dim3(256), 0, s, psi, count, value);
 }
 
 cudaError_t launch_minmax(const double *f, int64_t g, int64_t batch, MinMaxPart *part, int nblk,
@@ -450,11 +469,9 @@ cudaError_t launch_quantize(const double *f, uint32_t *fq, const InstDev *inst, 
 }
 
 cudaError_t launch_observables(const ObsArgs &a, int64_t batch, cudaStream_t s) {
-    k_obs_partial<<<dim3((unsigned)a.nblk, (unsigned)batch), 256, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_overlapped(true, k_obs_partial, dim3((unsigned)a.nblk, (unsigned)batch), dim3(256), 0, s, a);
     if (e != cudaSuccess) return e;
-    k_obs_final<<<(unsigned)batch, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(true, k_obs_final, dim3((unsigned)batch), dim3(256), 0, s, a);
 }
 
 void plan_of(int n, int *r1, int *r2) {

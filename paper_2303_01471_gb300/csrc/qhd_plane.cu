@@ -10,6 +10,7 @@
 //   then the local transforms with the kinetic phase in between.  psi touches
 //   global memory only at the chunk's start and end.
 #include "qhd_kernels.h"
+#include "qhd_launch.cuh"
 #include "qhd_plane.cuh"
 
 namespace qhd {
@@ -37,8 +38,8 @@ __global__ void __launch_bounds__(PLANE_THREADS, plane_min_blocks<N1, N2, C>()) 
     float2 *g = a.psi + plane * (int64_t)N1 * N2 + (int64_t)rank * P::R * N2;
     const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
 
-    plane_copy<N1, N2, C, true>(tile, g);
     const uint32_t *fqr = a.fq + plane * (int64_t)N1 * N2;
+    grid_release();
     {
         // the potential rows this CTA's exchange positions read (R / C rows in
         // each of the C row blocks) go to L2 now, during the tile load and the
@@ -50,6 +51,8 @@ __global__ void __launch_bounds__(PLANE_THREADS, plane_min_blocks<N1, N2, C>()) 
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(FQB) : "memory");
         }
     }
+    grid_wait();
+    plane_copy<N1, N2, C, true>(tile, g);
     load_phase_tab(ptab, a.ptab);
     const uint64_t coef = a.pot[plane / a.planes_per_inst];
     plane_copy_wait();
@@ -82,12 +85,13 @@ __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(PlaneArgs a
     uint32_t tiles[C];
 #pragma unroll
     for (int q = 0; q < C; ++q) tiles[q] = cluster_addr(tile, (uint32_t)q);
+    grid_release();
     plane_whole_run<N1, N2, C, 1>(a, blockIdx.x / C, rank, tiles, ptab, tile, true, cluster);
 }
 
 // ---------------------------------------------------------------- launchers
 template <typename K>
-static cudaError_t launch_cluster(K kernel, int64_t clusters, int c, size_t smem, const PlaneArgs &a,
+static cudaError_t launch_cluster(K kernel, bool overlap, int64_t clusters, int c, size_t smem, const PlaneArgs &a,
                                   cudaStream_t s, bool &attr_done) {
     if (!attr_done) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -99,13 +103,15 @@ static cudaError_t launch_cluster(K kernel, int64_t clusters, int c, size_t smem
     cfg.blockDim = dim3(PLANE_THREADS, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)c;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // kernels follow qhd_launch.cuh's rules
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
@@ -114,13 +120,13 @@ static cudaError_t launch_cluster(K kernel, int64_t clusters, int c, size_t smem
 template <int N1, int N2, int C>
 static cudaError_t plane_pass_impl(const PlaneArgs &a, cudaStream_t s) {
     static bool attr_done = false;
-    return launch_cluster(k_plane_pass<N1, N2, C>, a.planes, C, PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
+    return launch_cluster(k_plane_pass<N1, N2, C>, a.planes * N1 * N2 < OVERLAP_POINTS, a.planes, C, PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
 }
 
 template <int N1, int N2, int C, int MINB = 2>
 static cudaError_t plane_whole_impl(const PlaneArgs &a, cudaStream_t s) {
     static bool attr_done = false;
-    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, a.batch, C, PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
+    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, true, a.batch, C, PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
 }
 
 // Cluster size per distributed-axis length: R = 32 rows per CTA (16 for 32).

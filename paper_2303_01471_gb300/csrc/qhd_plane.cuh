@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "qhd_device.cuh"
+#include "qhd_launch.cuh"
 
 namespace qhd {
 
@@ -267,8 +268,9 @@ __device__ __forceinline__ void plane_whole_run(const PlaneArgs &a, int64_t b, i
     using P = PlaneCfg<N1, N2, C>;
     float2 *g = a.psi + b * (int64_t)N1 * N2 + (int64_t)rank * P::R * N2;
     const uint32_t *fqr = a.fq + b * (int64_t)N1 * N2;
-    if (live) plane_copy<N1, N2, C, true>(tile, g);
     load_phase_tab(ptab, a.ptab);
+    grid_wait();  // returns at once where the launch has nothing to overlap with
+    if (live) plane_copy<N1, N2, C, true>(tile, g);
     plane_copy_wait();
     cluster.sync();
 #pragma unroll 1

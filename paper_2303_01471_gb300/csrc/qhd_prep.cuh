@@ -16,12 +16,12 @@
 
 namespace qhd {
 
-// Potential coefficient pot[jl][b] (64-bit fraction of a turn per unit of the
-// fixed-point potential) and, for steps jl < cnt, the per-axis multipliers of
-// the kinetic phase: k_turns[d] (turns per unit m^2, 64-bit fraction) and
-// k_fd[d] (turns per unit sin^2(pi m / N)).
-__device__ inline void prep_coefficients(const PrepArgs &a, int64_t jl, int64_t b, uint64_t *k_turns,
-                                         double *k_fd, bool write_pot = true) {
+// Returns the potential coefficient pot[jl][b] (64-bit fraction of a turn per
+// unit of the fixed-point potential); for steps jl < cnt also gives the per-axis
+// multipliers of the kinetic phase: k_turns[d] (turns per unit m^2, 64-bit
+// fraction) and k_fd[d] (turns per unit sin^2(pi m / N)).
+__device__ inline uint64_t prep_coefficients(const PrepArgs &a, int64_t jl, int64_t b, uint64_t *k_turns,
+                                             double *k_fd) {
     const int64_t j = a.j0 + jl;  // global step index
     const SchedDev &sd = a.sched[b];
     const double PI = 3.141592653589793238462643383279502884;
@@ -44,7 +44,6 @@ __device__ inline void prep_coefficients(const PrepArgs &a, int64_t jl, int64_t 
     const int shift = a.inst[b].shift;
     // turns per unit of the fixed-point potential: theta / (2 pi) * 2^-shift
     const double y = ldexp(theta / (2.0 * PI), -shift);
-    if (write_pot) a.pot[jl * a.batch + b] = frac_to_u64(y);
     for (int d = 0; d < a.ndim; ++d) {
         // turns per unit m^2: dt * a * |2 pi m / L|^2 / 2 / (2 pi) = dt a pi m^2 / L^2
         const double kap = __ddiv_rn(__dmul_rn(__dmul_rn(a.dt, a_p), PI), __dmul_rn(a.len[d], a.len[d]));
@@ -53,13 +52,12 @@ __device__ inline void prep_coefficients(const PrepArgs &a, int64_t jl, int64_t 
         const double nn = (double)a.n[d];
         k_fd[d] = __ddiv_rn(__dmul_rn(__dmul_rn(a.dt, a_p), nn * nn), __dmul_rn(PI, __dmul_rn(a.len[d], a.len[d])));
     }
+    return frac_to_u64(y);
 }
 
-// Kinetic table entry i (axis d, mode m) of step jl and table row b:
+// Kinetic table entry i (axis d, mode m) of one step and instance:
 // exp(-2 pi i turns), times 1/G on axis 0, as an FP32 hi/lo pair.
-__device__ inline void prep_kinetic_entry(const PrepArgs &a, int64_t jl, int64_t b, int i, const uint64_t *k_turns,
-                                          const double *k_fd) {
-    float4 *out = a.kt + (jl * a.kt_batch + b) * a.ksum;
+__device__ inline float4 prep_kinetic_entry(const PrepArgs &a, int i, const uint64_t *k_turns, const double *k_fd) {
     int d = 0;
     while (d + 1 < a.ndim && i >= a.koff[d + 1]) ++d;
     const int idx = i - a.koff[d];
@@ -77,7 +75,7 @@ __device__ inline void prep_kinetic_entry(const PrepArgs &a, int64_t jl, int64_t
     const double scale = d == 0 ? a.inv_g : 1.0;  // exact power of two
     const double cr = c * scale, ci = -s * scale;
     const float hr = (float)cr, hi = (float)ci;
-    out[i] = make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
+    return make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
 }
 
 }  // namespace qhd
