@@ -253,13 +253,15 @@ qhd_status qhd_set_transform(qhd_ctx *ctx, int transform, int products, void *tc
  * tensor-core transform runs on this library's own GEMM kernel. */
 int64_t qhd_library_call_count(const qhd_ctx *ctx);
 
-/* CTAs per instance (2-D grids held in one thread-block cluster for a whole
- * chunk of steps) or per plane (3-D plane passes) of the cluster engine; 0 for
- * the generic passes or a NULL context.  For 2-D grids whose axis 0 has 64 or
- * 128 points, a batch with at most (SM count / wide split) instances runs on
- * twice the default CTAs per instance (4 for 64, 8 for 128: half the rows per
- * CTA), fixed at qhd_init_grid.  A batched group (qhd_group_*) uses the same
- * split by default. */
+/* CTAs per instance (2-D grids held on chip for a whole chunk of steps) or per
+ * plane (3-D plane passes) of the plane engine; 0 for the generic passes or a
+ * NULL context.  For 2-D grids whose axis 0 has 64 or 128 points, a batch with at
+ * most (SM count / wide split) instances runs on twice the default CTAs per
+ * instance (4 for 64, 8 for 128: half the rows per CTA).  Batches that fill the
+ * GPU several times over run their instances of up to 16384 points in one CTA
+ * each (reported as 1; what does not fill a wave may still run on clusters).
+ * Fixed at qhd_init_grid.  A batched group (qhd_group_*) uses the same split by
+ * default (128^2: never less than 4). */
 int qhd_cluster_ctas(const qhd_ctx *ctx);
 
 /*

@@ -8,7 +8,8 @@
 //     the same arithmetic as the stand-alone prep kernel, qhd_prep.cuh);
 //   * instance items run every Strang step of the chunk for CL / sub instances
 //     of one context, each held in the shared memory of `sub` CTAs of the
-//     cluster (the whole-run engine of qhd_plane.cuh).
+//     cluster (the whole-run engine of qhd_plane.cuh; sub = 1, for 64^2: the solo
+//     form of qhd_plane2.cuh).
 // All prep items precede all instance items in the queue, and a cluster claims
 // an item only when it has finished the previous one, so when an instance item
 // waits for its context's tables, every prep item it needs has been claimed by
@@ -30,6 +31,7 @@
 #include "qhd_trace.h"
 #include "qhd_kernels.h"
 #include "qhd_plane.cuh"
+#include "qhd_plane2.cuh"
 #include "qhd_prep.cuh"
 
 namespace qhd {
@@ -104,6 +106,17 @@ __device__ __forceinline__ void group_run(const PlaneArgs &pa, int64_t b, bool l
     plane_whole_run<N, N, C, 1>(pa, b, r, tiles, ptab, tile, live, cluster);
 }
 
+// One CTA per instance (solo form): nothing is shared between the CTAs, so an
+// idle one has nothing to do.
+template <int N>
+__device__ __noinline__ void group_solo(const PlaneArgs &pa, int64_t b, bool live, float2 *tile, float4 *ptab) {
+    using P = Solo<N, N>;
+    static_assert(P::THREADS == PLANE_THREADS, "one instance per CTA");
+    load_phase_tab(ptab, pa.ptab);
+    __syncthreads();
+    if (live) solo_whole_run<P>(pa, b, ptab, reinterpret_cast<ulonglong2 *>(tile), (int)threadIdx.x);
+}
+
 // Instance item k of context c: wait for its tables, then every step of the
 // chunk for instances k * (CL / sub) + grp, grp = 0 .. CL / sub - 1.
 __device__ __forceinline__ void group_instance(const GroupArgs &a, const GroupClass &g, int c, int64_t k, int crank,
@@ -132,6 +145,7 @@ __device__ __forceinline__ void group_instance(const GroupArgs &a, const GroupCl
     const bool live = b < s_pa.batch;
     const int64_t bb = live ? b : s_pa.batch - 1;  // idle CTAs read a valid instance's tables
     switch (g.n * 16 + sub) {
+    case 64 * 16 + 1: group_solo<64>(s_pa, bb, live, tile, ptab); break;
     case 64 * 16 + 2: group_run<64, 2>(s_pa, bb, live, grp, r, tile, ptab, cluster); break;
     case 64 * 16 + 4: group_run<64, 4>(s_pa, bb, live, grp, r, tile, ptab, cluster); break;
     case 64 * 16 + 8: group_run<64, 8>(s_pa, bb, live, grp, r, tile, ptab, cluster); break;
@@ -180,9 +194,10 @@ __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_group(GroupArgs a) {
     }
 }
 
-// Shared memory of one CTA for a (edge, CTAs per instance) class.
+// Shared memory of one CTA for a (edge, CTAs per instance) class; 0: no such class.
 static size_t class_smem(int n, int sub) {
     switch (n * 16 + sub) {
+    case 64 * 16 + 1: return Solo<64, 64>::SMEM;
     case 64 * 16 + 2: return PlaneCfg<64, 64, 2>::SMEM;
     case 64 * 16 + 4: return PlaneCfg<64, 64, 4>::SMEM;
     case 64 * 16 + 8: return PlaneCfg<64, 64, 8>::SMEM;
@@ -340,9 +355,12 @@ qhd_status qhd_group_create(qhd_group **out, qhd_ctx *const *ctxs, int n_ctx, co
             return QHD_ERR_INVALID_ARG;
         }
         const int idx = v.n[0] == 64 ? 0 : v.n[0] == 128 ? 1 : 2;
-        // default: the context's own split, so the group runs its arithmetic
-        const int sub = c.sub_cluster[idx] ? c.sub_cluster[idx] : (v.plane_c ? v.plane_c : default_sub(v.n[0]));
-        if (!sub_ok(v.n[0], sub)) {
+        // default: the context's own split, so the group runs its arithmetic; 128^2 in
+        // one CTA each wants 512 threads and an SM of its own, which the launch's
+        // clusters of two CTAs per SM do not give
+        int sub = c.sub_cluster[idx] ? c.sub_cluster[idx] : v.plane_c;
+        if (!c.sub_cluster[idx] && (sub == 0 || (sub == 1 && v.n[0] != 64))) sub = default_sub(v.n[0]);
+        if (c.sub_cluster[idx] == 1 || !sub_ok(v.n[0], sub)) {
             delete g;
             return QHD_ERR_INVALID_ARG;
         }
@@ -358,20 +376,10 @@ qhd_status qhd_group_create(qhd_group **out, qhd_ctx *const *ctxs, int n_ctx, co
     g->d_error = (unsigned *)(g->work + L.error);
     g->d_twx = (float4 *)(g->work + L.twx);
     // exchange twiddles of the distributed axis for the chosen split N = sub * R:
-    // twx[q * R + j] = exp(-2 pi i j q / N), FP32 hi/lo from FP64
     std::vector<float4> twx(GROUP_TWX * (size_t)n_ctx, make_float4(0.f, 0.f, 0.f, 0.f));
     for (int i = 0; i < n_ctx; ++i) {
         const int64_t n = g->edge[(size_t)i];
-        const int sub = g->sub[(size_t)i], rr = (int)n / sub;
-        for (int q = 0; q < sub; ++q)
-            for (int j = 0; j < rr; ++j) {
-                const double ang = 2.0 * 3.141592653589793238462643383279502884 *
-                                   (double)(((int64_t)j * q) % n) / (double)n;
-                const double cr = cos(ang), ci = -sin(ang);
-                const float hr = (float)cr, hi = (float)ci;
-                twx[(size_t)i * GROUP_TWX + (size_t)(q * rr + j)] =
-                    make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
-            }
+        exchange_twiddles(&twx[(size_t)i * GROUP_TWX], (int)n, g->sub[(size_t)i]);
     }
     void *kern = group_kernel(g->min_blocks);
     // a stream of the group's own: the caller's stream may be one that cannot be
@@ -488,6 +496,8 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
                 pl.pot = v.pot;
                 pl.kt = v.kt;
                 pl.tw_row = v.tw_row;
+                pl.tw_row2 = v.tw_row2;
+                pl.twc = v.twc;
                 pl.twx = g->d_twx + (size_t)i * GROUP_TWX;
                 pl.batch = v.batch;
                 pl.cnt = (int)cnt;

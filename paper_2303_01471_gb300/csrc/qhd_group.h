@@ -19,6 +19,7 @@ struct GroupCtxView {
     const uint32_t *fq;
     uint64_t *pot;           // [chunk + 1][batch]
     float4 *kt;              // [chunk][kt_batch][ksum]
+    const float4 *tw_row2, *twc;  // packed row twiddles, column twiddles of the solo form
     const float4 *tw_row;    // stage-2 twiddles of axis 1
     const float4 *ptab;
     const SchedDev *sched;

@@ -32,11 +32,18 @@ constexpr int MINMAX_BLOCKS_MAX = 512;
 size_t align_up(size_t v) { return (v + 255) & ~size_t(255); }
 
 struct Layout {
-    size_t f64, fq, kt, pot, sched, samples, inst, tw, twx, ptab, coord, obs_part, obs_res, mm, total;
+    size_t f64, fq, kt, pot, sched, samples, inst, tw, tw2, twx, twc, ptab, coord, obs_part, obs_res, mm, total;
     int64_t chunk;         // steps per chunk with one kinetic table per instance
     int64_t chunk_shared;  // steps per chunk when all instances share the kinetic table
     int obs_blocks, mm_blocks;
 };
+
+// log2 of a power of two
+int log2i(int64_t v) {
+    int k = 0;
+    while ((int64_t(1) << k) < v) ++k;
+    return k;
+}
 
 int64_t grid_points(int ndim, const int64_t *n) {
     int64_t g = 1;
@@ -93,7 +100,9 @@ Layout make_layout(int ndim, const int64_t *n, int64_t batch) {
     L.samples = take(sizeof(double) * 3 * MAX_TABLE_SAMPLES * (size_t)batch);
     L.inst = take(sizeof(InstDev) * (size_t)batch);
     L.tw = take(sizeof(float4) * (size_t)(ksum));
+    L.tw2 = take(sizeof(float4) * 2 * TW2_TABLE * (size_t)(ksum));
     L.twx = take(sizeof(float4) * (size_t)(ksum));
+    L.twc = take(sizeof(float4) * (size_t)(ksum));
     L.ptab = take(sizeof(float4) * (size_t)PHASE_TAB);
     L.coord = take(sizeof(double) * (size_t)ksum);
     L.obs_part = take(sizeof(double) * 3 * (size_t)L.obs_blocks * (size_t)batch);
@@ -125,10 +134,13 @@ struct qhd_ctx {
     double *samples = nullptr;
     InstDev *inst = nullptr;
     float4 *tw[3] = {nullptr, nullptr, nullptr};
+    float4 *tw2[3] = {nullptr, nullptr, nullptr};  // twiddles of the packed line FFT
     float4 *twx = nullptr;  // exchange twiddles of the cluster-distributed axis
+    float4 *twc = nullptr;  // column twiddles of the solo plane engine
     float4 *ptab = nullptr; // potential phase table exp(-2 pi i (k + 1/2) / PHASE_TAB), hi/lo
     int plane_mode = 0;     // 0 generic passes, 2 whole-run 2-D clusters, 3 3-D plane pass
-    int plane_c = 0;        // CTAs per instance (2-D) or per plane (3-D) of the cluster engine
+    int plane_c = 0;        // CTAs per instance (2-D) or per plane (3-D) of the plane engines
+    int64_t solo = 0;       // 2-D: the first `solo` instances run in one CTA each
     double *coord = nullptr;
     double *obs_part = nullptr, *obs_res = nullptr;
     MinMaxPart *mm = nullptr;
@@ -352,9 +364,34 @@ qhd_status qhd_init_grid(qhd_ctx **out, int ndim, const int64_t *n, const double
                     make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
             }
     }
+    // twiddles of the packed line FFT, both plans, one table per stage after the
+    // first: entry [m * L + j] = exp(-2 pi i j m / (L R)), L the product of the
+    // radices before the stage, R its radix
+    std::vector<float4> tw2((size_t)(2 * TW2_TABLE * c->ksum), make_float4(0.f, 0.f, 0.f, 0.f));
+    for (int d = 0; d < ndim; ++d) {
+        const size_t first = (size_t)(2 * TW2_TABLE) * (size_t)c->koff[d];
+        c->tw2[d] = (float4 *)(c->work + L.tw2) + first;
+        for (int v = 0; v < 2; ++v) {
+            int radix[4], stages = 0;
+            plan2_of((int)n[d], v, radix, &stages);
+            size_t at = first + (size_t)(v * TW2_TABLE) * (size_t)n[d];
+            int64_t l = radix[0];
+            for (int st = 1; st < stages; l *= radix[st], ++st) {
+                const int64_t period = l * radix[st];
+                for (int64_t i = 0; i < period; ++i) {
+                    const double ang = 2.0 * 3.141592653589793238462643383279502884 *
+                                       (double)(((i % l) * (i / l)) % period) / (double)period;
+                    const double cr = cos(ang), ci = -sin(ang);
+                    const float hr = (float)cr, hi = (float)ci;
+                    tw2[at++] = make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
+                }
+            }
+        }
+    }
     // cluster plane engine: 2-D grids with both axes in 32..256 stay resident in
     // one cluster per instance; 3-D grids whose last two axes fit use plane passes
     c->twx = (float4 *)(c->work + L.twx);
+    c->twc = (float4 *)(c->work + L.twc);
     int dist_axis = -1;
     if (ndim == 2 && plane_supported((int)n[0], (int)n[1])) {
         c->plane_mode = 2;
@@ -363,27 +400,36 @@ qhd_status qhd_init_grid(qhd_ctx **out, int ndim, const int64_t *n, const double
         // a batch that leaves most SMs idle runs each instance on twice the CTAs
         int dev = 0, sms = 0;
         const int wide = plane_cluster_wide((int)n[0]);
-        if (wide && cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-            batch * (int64_t)wide <= (int64_t)sms)
-            c->plane_c = wide;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
+            if (wide && batch * (int64_t)wide <= (int64_t)sms) {
+                c->plane_c = wide;
+            } else if (plane_fits_solo((int)n[0], (int)n[1])) {
+                // One CTA per instance for whole waves of the GPU; what is left over
+                // runs on clusters if those fill at most two CTAs per SM (128^2: a solo
+                // wave of 152 takes 18.6 us per step, 152 instances on clusters 26.6, but
+                // 60 instances 10.3; 64^2: 456 14.8 / 19.9, and 152 12.6 / 6.7).
+                // A single wave with a few instances left over gains too little to pay
+                // for the second launch (128^2 x 160: 28.5 us, on clusters 26.8).
+                const int64_t wave = (int64_t)sms * solo_per_sm((int)n[0], (int)n[1]);
+                const int64_t left = batch % wave;
+                c->solo = left * c->plane_c <= 2 * (int64_t)sms ? batch - left : batch;
+                if (c->solo == wave && left > 0 && 7 * left < wave) c->solo = 0;
+                if (c->solo > 0) c->plane_c = 1;
+            }
+        }
     }
     else if (ndim == 3 && plane_supported((int)n[1], (int)n[2])) {
         c->plane_mode = 3;
         dist_axis = 1;
-        c->plane_c = plane_cluster((int)n[1]);
+        c->plane_c = plane_fits_solo((int)n[1], (int)n[2]) ? 1 : plane_cluster((int)n[1]);
     }
     std::vector<float4> twx((size_t)c->ksum, make_float4(0.f, 0.f, 0.f, 0.f));
+    std::vector<float4> twc((size_t)c->ksum, make_float4(0.f, 0.f, 0.f, 0.f));
     if (dist_axis >= 0) {
-        const int n1 = (int)n[dist_axis], cc = c->plane_c, rr = n1 / cc;
-        for (int q = 0; q < cc; ++q)
-            for (int j = 0; j < rr; ++j) {
-                const double ang = 2.0 * 3.141592653589793238462643383279502884 * (double)(((int64_t)j * q) % n1) /
-                                   (double)n1;
-                const double cr = cos(ang), ci = -sin(ang);
-                const float hr = (float)cr, hi = (float)ci;
-                twx[(size_t)(q * rr + j)] = make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
-            }
+        if (ndim == 2) exchange_twiddles(twx.data(), (int)n[dist_axis], c->plane_c > 1 ? c->plane_c : plane_cluster((int)n[0]));
+        else exchange_twiddles2(twx.data(), (int)n[dist_axis], c->plane_c);
+        solo_twiddles(twc.data(), (int)n[dist_axis]);
     }
     // potential phase table
     c->ptab = (float4 *)(c->work + L.ptab);
@@ -403,7 +449,11 @@ qhd_status qhd_init_grid(qhd_ctx **out, int ndim, const int64_t *n, const double
     cudaError_t e = cudaMemcpyAsync(c->work + L.tw, tw.data(), tw.size() * sizeof(float4),
                                     cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->work + L.tw2, tw2.data(), tw2.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->twx, twx.data(), twx.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->twc, twc.data(), twc.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->ptab, ptab.data(), ptab.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
@@ -697,6 +747,8 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
             w.pot = c->pot;
             w.kt = c->kt;
             w.tw_row = c->tw[1];
+            w.tw_row2 = c->tw2[1];
+            w.twc = c->twc;
             w.twx = c->twx;
             w.batch = B;
             w.cnt = (int)cnt;
@@ -706,24 +758,31 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
             w.ptab = c->ptab;
             w.kt_batch = ktb;
             TimedScope ts(c, QHD_KCLASS_WHOLE, true);
-            if (c->plane_c == plane_cluster((int)c->n[0]))
-                QHD_LAUNCH(c, launch_plane_whole((int)c->n[0], (int)c->n[1], w, c->stream));
-            else
-                QHD_LAUNCH(c, launch_plane_whole_wide((int)c->n[0], (int)c->n[1], w, c->stream));
+            w.instances = c->solo;
+            if (c->solo > 0) QHD_LAUNCH(c, launch_solo_whole((int)c->n[0], (int)c->n[1], w, c->stream));
+            w.first = c->solo;
+            w.instances = B - c->solo;
+            if (w.instances > 0) {
+                if (c->plane_c == plane_cluster_wide((int)c->n[0]))
+                    QHD_LAUNCH(c, launch_plane_whole_wide((int)c->n[0], (int)c->n[1], w, c->stream));
+                else
+                    QHD_LAUNCH(c, launch_plane_whole((int)c->n[0], (int)c->n[1], w, c->stream));
+            }
             continue;
         }
         const int last_ax = ndim - 1;
         RowArgs r{};
         r.psi = c->psi;
         r.fq = c->fq;
-        r.tw2 = c->tw[last_ax];
+        r.tw2 = c->tw2[last_ax];
         r.rows = B * (c->g / c->n[last_ax]);
-        r.rows_per_inst = c->g / c->n[last_ax];
+        r.log_rows = log2i(c->g / c->n[last_ax]);
         r.ptab = c->ptab;
         AxisArgs ax0{};
         ax0.psi = c->psi;
-        ax0.tw2 = c->tw[0];
+        ax0.tw2 = c->tw2[0];
         ax0.inner = c->g / c->n[0];
+        ax0.log_inner = log2i(ax0.inner);
         ax0.planes = B;
         ax0.ksum = c->ksum;
         ax0.koff1 = c->koff[1];
@@ -736,21 +795,24 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
         if (c->plane_mode == 3) {
             pl.psi = c->psi;
             pl.fq = c->fq;
-            pl.tw_row = c->tw[2];
+            pl.tw_row2 = c->tw2[2];
+            pl.twc = c->twc;
             pl.twx = c->twx;
             pl.planes = B * c->n[0];
-            pl.planes_per_inst = c->n[0];
+            pl.log_planes = log2i(c->n[0]);
             pl.batch = B;
             pl.ptab = c->ptab;
-            const int cc = plane_cluster((int)c->n[1]);
-            ax0.perm1_r = (int)c->n[1] / cc;
-            ax0.perm1_c = cc;
+            // rows of a plane that one CTA holds keep their natural frequency order
+            const int cc = c->plane_c;
+            ax0.perm1_log_r = log2i(c->n[1] / cc);
+            ax0.perm1_c = cc > 1 ? cc : 0;
         }
         AxisArgs ax1{};
         if (ndim == 3) {
             ax1.psi = c->psi;
-            ax1.tw2 = c->tw[1];
+            ax1.tw2 = c->tw2[1];
             ax1.inner = c->n[2];
+            ax1.log_inner = log2i(ax1.inner);
             ax1.planes = B * c->n[0];
             ax1.ndim = ndim;
         }
@@ -1062,6 +1124,8 @@ qhd_status ctx_group_view(qhd_ctx *c, GroupCtxView *v) {
     v->pot = c->pot;
     v->kt = c->kt;
     v->tw_row = c->ndim >= 2 ? c->tw[1] : nullptr;
+    v->tw_row2 = c->ndim >= 2 ? c->tw2[1] : nullptr;
+    v->twc = c->twc;
     v->ptab = c->ptab;
     v->sched = c->sched;
     v->inst = c->inst;

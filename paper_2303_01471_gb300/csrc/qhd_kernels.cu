@@ -20,9 +20,12 @@
 // turn per unit of f; the kinetic phase uses integer m^2 and a 64-bit fraction
 // of a turn per unit of m^2.  The product modulo one turn is exact to 2^-32,
 // so the FP32 sine/cosine only ever sees a reduced argument.
+#include <type_traits>
+
 #include "qhd_device.cuh"
 #include "qhd_kernels.h"
 #include "qhd_launch.cuh"
+#include "qhd_packed.cuh"
 #include "qhd_sched.cuh"
 #include "qhd_prep.cuh"
 
@@ -37,123 +40,152 @@ struct BlockSync {
 
 constexpr int ROW_THREADS = 128;
 
-__host__ __device__ constexpr int axis_w(int n) {
-    // columns per tile of a strided pass: 32-byte row segments at least,
-    // 128 threads per block
-    return n >= 1024 ? 4 : n >= 256 ? 8 : n >= 64 ? 16 : 32;
-}
+// The row and axis passes work on pairs of lines in packed FP32
+// (qhd_packed.cuh): rows 2i and 2i + 1, columns 2i and 2i + 1.  Every axis
+// length is even, so the pairs never straddle an instance or a plane.
 
 // --------------------------------------------------------------- row pass
-template <int N>
-__global__ void __launch_bounds__(ROW_THREADS) k_row(RowArgs a) {
-    using C = LineCfg<N>;
+template <int N, int V>
+__global__ void __launch_bounds__(ROW_THREADS, 4) k_row(RowArgs a) {
+    using C = Line2<N, V>;
+    using B = RowBuf<N, V>;
+    const RowAddr<C::LOG_R1> at;
     constexpr int E = C::E, T = C::T;
-    constexpr int S = line_stride<N>(true, 0);
+    using Sync = std::conditional_t<(T > 32), BlockSync, WarpSync>;
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
-    float2 *smem = reinterpret_cast<float2 *>(smem4 + PHASE_TAB);
     grid_release();
     load_phase_tab(ptab, a.ptab);
     __syncthreads();
-    grid_wait();
-    const int lpb = blockDim.x / T;
     const int line = threadIdx.x / T, t = threadIdx.x % T;
-    const int64_t row = (int64_t)blockIdx.x * lpb + line;
+    const int64_t row = 2 * ((int64_t)blockIdx.x * (blockDim.x / T) + line);
     const bool valid = row < a.rows;
     const int64_t r = valid ? row : 0;
     float2 *g = a.psi + r * N;
     const uint32_t *fq = a.fq + r * N;
-    float2 x[E];
+    grid_wait();
+    c2 x[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) x[e] = g[t + T * e];
-    float2 *sm = smem + (C::TWO_STAGE ? line * S : 0);
-    if (a.mode & MODE_INV) line_fft<N, true>(x, sm, t, a.tw2, WarpSync{});
-    const uint64_t c = a.pot[r / a.rows_per_inst];
+    for (int e = 0; e < E; ++e) x[e] = c2_make(g[t + T * e], g[N + t + T * e]);
+    ulonglong2 *sm = reinterpret_cast<ulonglong2 *>(smem4 + PHASE_TAB) + line * B::S;
+    const float4 *tw = a.tw2;
+    if (a.mode & MODE_INV) line_fft2<N, V, true>(x, sm, t, tw, Sync{}, at);
+    const uint64_t c = a.pot[r >> a.log_rows];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        x[e] = apply_phase_tab(x[e], turns_mul(c, __ldg(&fq[t + T * e])) + a.dither, ptab);
+        const int i = t + T * e;
+        x[e] = apply_phase_tab2(x[e], turns_mul(c, __ldg(&fq[i])) + a.dither, turns_mul(c, __ldg(&fq[N + i])) + a.dither,
+                                ptab);
     }
-    if (a.mode & MODE_FWD) line_fft<N, false>(x, sm, t, a.tw2, WarpSync{});
+    if (a.mode & MODE_FWD) line_fft2<N, V, false>(x, sm, t, tw, Sync{}, at);
     if (valid) {
 #pragma unroll
-        for (int e = 0; e < E; ++e) g[t + T * e] = x[e];
+        for (int e = 0; e < E; ++e) {
+            g[t + T * e] = c2_first(x[e]);
+            g[N + t + T * e] = c2_second(x[e]);
+        }
     }
 }
 
 // ------------------------------------------------------ strided axis pass
-// Lines of length N at stride `inner`; a block owns W adjacent lines (columns)
-// of one plane, lanes run along the columns so each global access moves W
-// consecutive complex values per row.
-// Strided passes over lines up to 256 points are compiled for 4 resident blocks
-// per SM (issue-bound, latency hidden by warps); longer lines keep their
-// registers (32 points per thread).
-template <int N, int W>
-__global__ void __launch_bounds__(W * LineCfg<N>::T, N <= 256 ? 4 : 1) k_axis(AxisArgs a) {
-    using C = LineCfg<N>;
+// Lines of length N at stride `inner`; a block owns CP adjacent pairs of columns
+// of one plane, lanes run along the pairs, so each 16-byte access moves both
+// columns of a pair and each row of a tile is 16 CP contiguous bytes.
+// Resident blocks: 4 of 128 threads with 8 points per thread; 3 with 16 (at 4,
+// the 128 registers a thread may then use spill: 256^3 axis-0 pass 69 us, 66 at 3).
+template <int N, int V, int CP> constexpr int axis_min_blocks() {
+    constexpr int threads = CP * Line2<N, V>::T;
+    return threads < 128 ? 1 : (Line2<N, V>::E == 16 ? 3 : 4) * 128 / threads;
+}
+
+template <int N, int V, int CP>
+__global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>()) k_axis(AxisArgs a) {
+    using C = Line2<N, V>;
+    using B = ColBuf<N, V, CP>;
+    const ColBufAddr<N, V, CP> at;
     constexpr int E = C::E, T = C::T;
-    constexpr int S = line_stride<N>(false, W);
-    extern __shared__ float2 smem[];
-    const int c = threadIdx.x % W, t = threadIdx.x / W;
-    const int64_t tiles = a.inner / W;
-    const int64_t o = blockIdx.x / tiles;
-    const int64_t ci = (blockIdx.x - o * tiles) * W + c;
-    float2 *g = a.psi + o * (int64_t)N * a.inner + ci;
+    extern __shared__ __align__(16) float4 smem4[];
+    const int c = threadIdx.x % CP, t = threadIdx.x / CP;
+    constexpr int LOG_W = CP == 32 ? 6 : CP == 16 ? 5 : CP == 8 ? 4 : CP == 4 ? 3 : CP == 2 ? 2 : 1;  // log2(2 CP)
+    static_assert(1 << LOG_W == 2 * CP, "tile width");
+    const int64_t o = blockIdx.x >> (a.log_inner - LOG_W);
+    const int64_t tile = blockIdx.x - (o << (a.log_inner - LOG_W));
+    const int64_t ci = tile * (2 * CP) + 2 * c;
+    float4 *g = reinterpret_cast<float4 *>(a.psi + o * (int64_t)N * a.inner + ci);
+    const int64_t stride = a.inner / 2;
     grid_release();
     grid_wait();
-    float2 x[E];
+    c2 x[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) x[e] = g[(int64_t)(t + T * e) * a.inner];
-    float2 *sm = smem + (C::TWO_STAGE ? c * S : 0);
+    for (int e = 0; e < E; ++e) {
+        const float4 v = g[(int64_t)(t + T * e) * stride];
+        x[e] = c2_make(make_float2(v.x, v.y), make_float2(v.z, v.w));
+    }
+    ulonglong2 *sm = reinterpret_cast<ulonglong2 *>(smem4) + c * B::S;
+    const float4 *tw = a.tw2;
     // zero-mode split (qhd_device.cuh) in the forward-kinetic-inverse pass, for
     // the tile holding column 0 (frequency 0 of the other axes) of each
     // instance: the T threads of a column span several warps, so their partial
-    // sums meet in shared memory behind the exchange buffer and every thread
-    // adds them in the same order.
+    // sums meet in the exchange buffer's space and every thread adds them in the
+    // same order.  The sum, later its part of the result, waits in a slot behind
+    // the buffer, so that no other tile's pass holds registers for it.
     constexpr int ALL3 = MODE_FWD | MODE_KIN | MODE_INV;
-    const bool split0 = (a.mode & ALL3) == ALL3 && blockIdx.x == o * tiles;
-    float2 sum = make_float2(0.f, 0.f), mean_part = make_float2(0.f, 0.f);
+    const bool split0 = (a.mode & ALL3) == ALL3 && tile == 0;
+    ulonglong2 *slot = reinterpret_cast<ulonglong2 *>(smem4) + (C::STAGES > 1 ? CP * B::S : 0) + c;
     if (split0) {
-        float2 *red = smem + (C::TWO_STAGE ? W * S : 0);
-        float2 s = x[0];
+        ulonglong2 *red = reinterpret_cast<ulonglong2 *>(smem4);
+        c2 s = x[0];
 #pragma unroll
-        for (int e = 1; e < E; ++e) s = cadd(s, x[e]);
-        red[t * W + c] = s;
-        __syncthreads();
-        sum = red[c];
+        for (int e = 1; e < E; ++e) s = s + x[e];
+        if (T > 1) {
+            st_c2(&red[t * CP + c], s);
+            __syncthreads();
+            s = ld_c2(&red[c]);
+#pragma unroll 1
+            for (int q = 1; q < T; ++q) s = s + ld_c2(&red[q * CP + c]);
+            __syncthreads();
+        }
+        const c2 mu{s.x * pf_dup(1.0f / N), s.y * pf_dup(1.0f / N)};
 #pragma unroll
-        for (int q = 1; q < T; ++q) sum = cadd(sum, red[q * W + c]);
-        sub_line_mean<N, E>(x, sum);
+        for (int e = 0; e < E; ++e) x[e] = x[e] - mu;
+        if (t == 0) st_c2(slot, s);
     }
-    if (a.mode & MODE_FWD) line_fft<N, false>(x, sm, t, a.tw2, BlockSync{});
+    if (a.mode & MODE_FWD) line_fft2<N, V, false>(x, sm, t, tw, BlockSync{}, at);
     if (a.mode & MODE_KIN) {
-        // axis 0 pass: plane index o is the instance.  Each per-axis factor is
-        // an FP32 hi/lo pair applied with a compensated product: a table entry
-        // is shared by every point with the same frequency index, so a plain
-        // FP32 rounding of it would perturb the norm coherently.
+        // axis 0 pass: plane index o is the instance.  The per-axis factors are
+        // FP32 hi/lo pairs applied with compensated products: a table entry is
+        // shared by every point with the same frequency index, so a plain FP32
+        // rounding of it would perturb the norm coherently.  The factors of axes 1
+        // and 2 are the same for the whole column: their product (hi/lo again) is
+        // formed once.
         const float4 *kb = a.kt + (a.kt_batch == 1 ? 0 : o) * a.ksum;
-        int64_t i1 = a.ndim == 2 ? ci : (ci >> a.log_n2);
-        if (a.perm1_r) i1 = i1 / a.perm1_r + (int64_t)a.perm1_c * (i1 % a.perm1_r);
-        const float4 k1 = __ldg(&kb[a.koff1 + i1]);
-        float4 k2 = make_float4(1.f, 0.f, 0.f, 0.f);
-        if (a.ndim == 3) k2 = __ldg(&kb[a.koff2 + (ci & ((1 << a.log_n2) - 1))]);
-        auto kin = [&](float2 v, float4 k0) {
-            float2 y = cmul_comp(v, make_float2(k0.x, k0.y), make_float2(k0.z, k0.w));
-            y = cmul_comp(y, make_float2(k1.x, k1.y), make_float2(k1.z, k1.w));
-            if (a.ndim == 3) y = cmul_comp(y, make_float2(k2.x, k2.y), make_float2(k2.z, k2.w));
-            return y;
-        };
+        w2 kc;
+        if (a.ndim == 2) {
+            kc = w2_make(__ldg(&kb[a.koff1 + ci]), __ldg(&kb[a.koff1 + ci + 1]));
+        } else {
+            int64_t i1 = ci >> a.log_n2;
+            const int i2 = (int)(ci & ((1 << a.log_n2) - 1));
+            if (a.perm1_c) i1 = (i1 >> a.perm1_log_r) + a.perm1_c * (i1 & ((1 << a.perm1_log_r) - 1));
+            const float4 k1 = __ldg(&kb[a.koff1 + i1]);
+            kc = w2_mul(w2_make(k1, k1), w2_make(__ldg(&kb[a.koff2 + i2]), __ldg(&kb[a.koff2 + i2 + 1])));
+        }
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[e] = kin(x[e], __ldg(&kb[t + T * e]));
+        for (int e = 0; e < E; ++e) x[e] = c2_mul<false>(c2_mul_shared<false>(x[e], __ldg(&kb[t + T * e])), kc);
         // the mean's part: N mu = sum through the factor of frequency 0
-        if (split0) mean_part = kin(sum, __ldg(&kb[0]));
+        if (split0 && t == 0) st_c2(slot, c2_mul<false>(c2_mul_shared<false>(ld_c2(slot), __ldg(&kb[0])), kc));
     }
-    if (a.mode & MODE_INV) line_fft<N, true>(x, sm, t, a.tw2, BlockSync{});
+    if (a.mode & MODE_INV) line_fft2<N, V, true>(x, sm, t, tw, BlockSync{}, at);
     if (split0) {
+        // written by the column's thread 0 before the inverse transform's barriers
+        const c2 mean_part = ld_c2(slot);
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[e] = cadd(x[e], mean_part);
+        for (int e = 0; e < E; ++e) x[e] = x[e] + mean_part;
     }
 #pragma unroll
-    for (int e = 0; e < E; ++e) g[(int64_t)(t + T * e) * a.inner] = x[e];
+    for (int e = 0; e < E; ++e) {
+        const float2 p = c2_first(x[e]), q = c2_second(x[e]);
+        g[(int64_t)(t + T * e) * stride] = make_float4(p.x, p.y, q.x, q.y);
+    }
 }
 
 // --------------------------------------------- 1-D: a whole chunk per launch
@@ -382,35 +414,63 @@ __global__ void k_obs_final(ObsArgs a) {
 }
 
 // ---------------------------------------------------------------- launchers
-template <int N>
-static cudaError_t row_impl(const RowArgs &a, cudaStream_t s) {
-    using C = LineCfg<N>;
-    constexpr int S = line_stride<N>(true, 0);
-    const int lpb = ROW_THREADS / C::T;
-    const int64_t blocks = (a.rows + lpb - 1) / lpb;
-    const size_t sm = PHASE_TAB * sizeof(float4) + (C::TWO_STAGE ? (size_t)lpb * S * sizeof(float2) : 0);
-    return launch_overlapped(a.rows * N < OVERLAP_POINTS, k_row<N>, dim3((unsigned)blocks), dim3(ROW_THREADS), sm, s, a);
+template <int N, int V>
+static cudaError_t row_v_impl(const RowArgs &a, cudaStream_t s) {
+    using C = Line2<N, V>;
+    constexpr int PAIRS = ROW_THREADS / C::T;
+    const int64_t blocks = (a.rows / 2 + PAIRS - 1) / PAIRS;
+    constexpr size_t sm =
+        PHASE_TAB * sizeof(float4) + (C::STAGES > 1 ? (size_t)PAIRS * RowBuf<N, V>::S * sizeof(ulonglong2) : 0);
+    static_assert(sm <= 48 * 1024, "default shared-memory limit");
+    RowArgs r = a;
+    r.tw2 += V * TW2_TABLE * N;
+    return launch_overlapped(a.rows * N < OVERLAP_POINTS, k_row<N, V>, dim3((unsigned)blocks), dim3(ROW_THREADS), sm, s, r);
 }
 
-template <int N, int W>
-static cudaError_t axis_w_impl(const AxisArgs &a, cudaStream_t s) {
-    using C = LineCfg<N>;
-    constexpr int S = line_stride<N>(false, W);
-    const int64_t blocks = a.planes * (a.inner / W);
-    // exchange buffer, then the column partial sums of the zero-mode split
-    const size_t xch = (C::TWO_STAGE ? (size_t)W * S * sizeof(float2) : 0) + (size_t)W * C::T * sizeof(float2);
-    return launch_overlapped(a.planes * a.inner * N < OVERLAP_POINTS, k_axis<N, W>, dim3((unsigned)blocks), dim3(W * C::T), xch, s, a);
+template <int N>
+static cudaError_t row_impl(const RowArgs &a, cudaStream_t s) {
+    if constexpr (two_plans(N))
+        if (a.rows * N > BIG_PLAN_POINTS) return row_v_impl<N, 1>(a, s);
+    return row_v_impl<N, 0>(a, s);
+}
+
+// Pairs of columns per tile of a strided pass: 128 threads per block, at most
+// 32 pairs (512-byte row segments); 256 threads at 512 points, where 2 pairs are
+// only 32 bytes of each row (512^2 x 64 188 us per step, 183 with 4 pairs).
+__host__ __device__ constexpr int axis_cp(int n, int t) {
+    return n == 512 ? 4 : t >= 64 ? 2 : 128 / t > 32 ? 32 : 128 / t;
+}
+
+template <int N, int V, int CP>
+static cudaError_t axis_cp_impl(const AxisArgs &a, cudaStream_t s) {
+    using C = Line2<N, V>;
+    const int64_t blocks = a.planes * (a.inner / (2 * CP));
+    // exchange buffer (the zero-mode split's CP T partial sums use it too), then
+    // that split's slot per pair
+    constexpr size_t xch = ((C::STAGES > 1 ? (size_t)CP * ColBuf<N, V, CP>::S : 0) + CP) * sizeof(ulonglong2);
+    static_assert(xch <= 48 * 1024, "default shared-memory limit");
+    AxisArgs r = a;
+    r.tw2 += V * TW2_TABLE * N;
+    return launch_overlapped(a.planes * a.inner * N < OVERLAP_POINTS, k_axis<N, V, CP>, dim3((unsigned)blocks),
+                             dim3(CP * C::T), xch, s, r);
+}
+
+template <int N, int V>
+static cudaError_t axis_v_impl(const AxisArgs &a, cudaStream_t s) {
+    constexpr int CP = axis_cp(N, Line2<N, V>::T);
+    if (a.inner >= 2 * CP) return axis_cp_impl<N, V, CP>(a, s);
+    if constexpr (CP > 16) if (a.inner >= 32) return axis_cp_impl<N, V, 16>(a, s);
+    if constexpr (CP > 8) if (a.inner >= 16) return axis_cp_impl<N, V, 8>(a, s);
+    if constexpr (CP > 4) if (a.inner >= 8) return axis_cp_impl<N, V, 4>(a, s);
+    if constexpr (CP > 2) if (a.inner >= 4) return axis_cp_impl<N, V, 2>(a, s);
+    return axis_cp_impl<N, V, 1>(a, s);
 }
 
 template <int N>
 static cudaError_t axis_impl(const AxisArgs &a, cudaStream_t s) {
-    constexpr int WD = axis_w(N);
-    if (a.inner >= WD) return axis_w_impl<N, WD>(a, s);
-    if constexpr (WD > 16) if (a.inner >= 16) return axis_w_impl<N, 16>(a, s);
-    if constexpr (WD > 8) if (a.inner >= 8) return axis_w_impl<N, 8>(a, s);
-    if constexpr (WD > 4) if (a.inner >= 4) return axis_w_impl<N, 4>(a, s);
-    if (a.inner >= 2) return axis_w_impl<N, 2>(a, s);
-    return axis_w_impl<N, 1>(a, s);
+    if constexpr (two_plans(N))
+        if (a.planes * a.inner * N > BIG_PLAN_POINTS) return axis_v_impl<N, 1>(a, s);
+    return axis_v_impl<N, 0>(a, s);
 }
 
 template <int N>
@@ -472,6 +532,21 @@ cudaError_t launch_observables(const ObsArgs &a, int64_t batch, cudaStream_t s) 
     cudaError_t e = launch_overlapped(true, k_obs_partial, dim3((unsigned)a.nblk, (unsigned)batch), dim3(256), 0, s, a);
     if (e != cudaSuccess) return e;
     return launch_overlapped(true, k_obs_final, dim3((unsigned)batch), dim3(256), 0, s, a);
+}
+
+template <int N> static void plan2_radix(int v, int *radix, int *stages) {
+    for (int k = 0; k < 4; ++k) radix[k] = v ? Plan2<N, 1>::R[k] : Plan2<N, 0>::R[k];
+    *stages = v ? Line2<N, 1>::STAGES : Line2<N, 0>::STAGES;
+}
+void plan2_of(int n, int v, int *radix, int *stages) {
+    switch (n) {
+#define QHD_PLAN2_CASE(N) \
+    case N: return plan2_radix<N>(v, radix, stages);
+        QHD_PLAN2_CASE(2) QHD_PLAN2_CASE(4) QHD_PLAN2_CASE(8) QHD_PLAN2_CASE(16) QHD_PLAN2_CASE(32)
+        QHD_PLAN2_CASE(64) QHD_PLAN2_CASE(128) QHD_PLAN2_CASE(256) QHD_PLAN2_CASE(512) QHD_PLAN2_CASE(1024)
+#undef QHD_PLAN2_CASE
+    default: *stages = 0;
+    }
 }
 
 void plan_of(int n, int *r1, int *r2) {

@@ -37,9 +37,9 @@ struct RowArgs {
     float2 *psi;
     const uint32_t *fq;
     const uint64_t *pot;   // potential coefficient of this pass, one per instance
-    const float4 *tw2;
+    const float4 *tw2;     // twiddles of the row length (line_fft2), both plans
     int64_t rows;          // batch * rows per instance
-    int64_t rows_per_inst;
+    int log_rows;          // log2 of the rows per instance
     int mode;              // MODE_INV: inverse FFT before the phase; MODE_FWD: forward after
     uint32_t dither;       // global phase of this pass in 2^-32 turns (step_dither)
     const float4 *ptab;    // potential phase table (PHASE_TAB hi/lo entries)
@@ -47,9 +47,10 @@ struct RowArgs {
 
 struct AxisArgs {
     float2 *psi;
-    const float4 *tw2;
+    const float4 *tw2;     // twiddles of the line length (line_fft2), both plans
     const float4 *kt;      // kinetic tables of this step: [batch][ksum] (MODE_KIN only)
     int64_t inner;         // product of the axis lengths after this axis (line stride)
+    int log_inner;         // its log2
     int64_t planes;        // product of batch and the axis lengths before this axis
     int ksum;              // sum of the axis lengths
     int koff1, koff2;      // table offsets of axes 1 and 2
@@ -57,8 +58,8 @@ struct AxisArgs {
     int ndim;
     int mode;
     int64_t kt_batch;      // 1: every instance shares the kinetic table; else batch
-    int perm1_r, perm1_c;  // 3-D after a plane pass: stored axis-1 row s holds
-                           // frequency s / perm1_r + perm1_c * (s % perm1_r); 0 = natural
+    int perm1_log_r, perm1_c;  // 3-D after a plane pass: stored axis-1 row s holds frequency
+                               // s / r + perm1_c * (s % r), r = 2^perm1_log_r; perm1_c = 0: natural
 };
 
 // Plane engine (qhd_plane.cu): N1 distributed over a cluster, N2 per row.
@@ -67,11 +68,14 @@ struct PlaneArgs {
     const uint32_t *fq;
     const uint64_t *pot;     // pass: coefficients of this pass [batch]; whole: chunk [cnt+1][batch]
     const float4 *kt;        // whole: chunk kinetic tables [cnt][batch][ksum]
-    const float4 *tw_row;    // stage-2 twiddles of the row length
-    const float4 *twx;       // exchange twiddles twx[q*R + n2] = exp(-2 pi i n2 q / N1), (hi, lo)
+    const float4 *tw_row;    // cluster whole run: stage-2 twiddles of the row length (line_fft)
+    const float4 *tw_row2;   // others: twiddles of the row length (line_fft2), both plans
+    const float4 *twx;       // exchange twiddles: exchange_twiddles (whole), exchange_twiddles2 (pass)
+    const float4 *twc;       // solo form: column twiddles (solo_twiddles)
     int64_t planes;          // pass: batch * n0 planes
-    int64_t planes_per_inst; // pass: n0
+    int log_planes;          // pass: log2 of the planes per instance (n0)
     int64_t batch;
+    int64_t first, instances; // whole: the instances of this launch
     int mode;                // pass: MODE_INV (previous step's inverse first), MODE_FWD
     uint32_t dither;         // pass: global phase of this step
     int cnt;                 // whole: steps in the chunk
@@ -144,14 +148,28 @@ cudaError_t launch_quantize(const double *f, uint32_t *fq, const InstDev *inst, 
 cudaError_t launch_observables(const ObsArgs &a, int64_t batch, cudaStream_t s);
 cudaError_t launch_plane_pass(int n1, int n2, const PlaneArgs &a, cudaStream_t s);
 cudaError_t launch_plane_whole(int n1, int n2, const PlaneArgs &a, cudaStream_t s);
+cudaError_t launch_solo_whole(int n1, int n2, const PlaneArgs &a, cudaStream_t s);
 bool plane_supported(int n1, int n2);
+bool plane_fits_solo(int n1, int n2);  // one CTA holds the plane
+int solo_per_sm(int n1, int n2);       // instances an SM runs at once in the solo form
 int plane_cluster(int n1);
 // Whole-run kernel with twice the CTAs per instance (distributed axis 64 or 128; 0: none).
 int plane_cluster_wide(int n1);
 cudaError_t launch_plane_whole_wide(int n1, int n2, const PlaneArgs &a, cudaStream_t s);
 
 // Plans shared with the host (twiddle tables are built on the host).
-void plan_of(int n, int *r1, int *r2);
+void plan_of(int n, int *r1, int *r2);         // scalar line FFT (line_fft)
+void plan2_of(int n, int v, int *radix, int *stages);  // packed line FFT (line_fft2), plan v
+constexpr int TW2_TABLE = 2;  // table of plan v starts at v * TW2_TABLE * N; each holds at most TW2_TABLE * N entries
 bool supported_n(int64_t n);
+// Exchange twiddles of a distributed axis of n1 = c * r points, n1 entries:
+// exp(-2 pi i q j / n1) at [q * r + j], (re, im, residuals).
+void exchange_twiddles(float4 *out, int n1, int c);
+// The same for pairs of rows j = 2p, 2p + 1: values (re, re, im, im) at
+// [q * r / 2 + p], their FP32 residuals n1 / 2 entries later.
+void exchange_twiddles2(float4 *out, int n1, int c);
+// Column twiddles of the solo form, n1 entries: exp(-2 pi i k / n1), k < n1 / 2,
+// then the stage twiddles of a line of n1 / 2 points.
+void solo_twiddles(float4 *out, int n1);
 
 }  // namespace qhd

@@ -1,76 +1,111 @@
-// qhd_plane.cu -- kernels built on the cluster-resident plane engine.
+// qhd_plane.cu -- kernels built on the plane engines.
 //
-// k_plane_pass: one fused pass over the last two axes of a 3-D grid (for
-//   every (instance, i0) plane): inverse transform of the previous step along
+// k_solo_pass, k_plane_pass: one fused pass over the last two axes of a 3-D grid
+//   (for every (instance, i0) plane): inverse transform of the previous step along
 //   axes 2 and 1, potential phase, forward transform along axes 1 and 2.  With
 //   the axis-0 pass (forward, kinetic phase, inverse) a 3-D Strang step then
-//   reads and writes psi twice instead of four times.
-// k_plane_whole: a whole 2-D instance resident in one cluster for every step
-//   of a chunk: per step the cross-cluster exchange with the potential phase,
-//   then the local transforms with the kinetic phase in between.  psi touches
-//   global memory only at the chunk's start and end.
+//   reads and writes psi twice instead of four times.  Planes of up to 16384
+//   points take one CTA each, larger ones a cluster.
+// k_solo_whole, k_plane_whole: a whole 2-D instance resident in one CTA or one
+//   cluster for every step of a chunk: per step the potential phase between the
+//   column transforms and the kinetic phase between the row transforms.  psi
+//   touches global memory only at the chunk's start and end.
+#include <cmath>
+
 #include "qhd_kernels.h"
 #include "qhd_launch.cuh"
 #include "qhd_plane.cuh"
+#include "qhd_plane2.cuh"
 
 namespace qhd {
 
-// Resident CTAs per SM the pass is compiled for: as many as the tile's shared
-// memory allows, at most 3 (the pass is issue-bound; more warps hide latency).
-template <int N1, int N2, int C> constexpr int plane_min_blocks() {
-    constexpr size_t smem = PlaneCfg<N1, N2, C>::SMEM;
-    constexpr int by_smem = (int)((227 * 1024) / smem);
-    return by_smem >= 3 ? 3 : by_smem < 1 ? 1 : by_smem;
+// Resident CTAs per SM a kernel on pairs of rows is compiled for: 512 threads of
+// 128 registers where one holds 16 pairs of points, 768 of 80 where it holds 8
+// (64^3 x 32 84.4 us per step, 90.3 with 512 threads, 86.6 with 1024), or what the
+// tiles' shared memory allows.
+template <typename P> constexpr int plane2_min_blocks(int threads) {
+    constexpr int by_smem = (int)((227 * 1024) / (P::SMEM + 1024));
+    const int by_regs = threads / P::THREADS < 1 ? 1 : threads / P::THREADS;
+    return by_smem < by_regs ? by_smem : by_regs;
+}
+template <typename P> constexpr int solo_min_blocks() {
+    return plane2_min_blocks<P>(P::E2 == 16 || P::RP == 64 ? 512 : 768);
+}
+
+template <int N1, int N2>
+__global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1, N2>>()) k_solo_pass(PlaneArgs a) {
+    using P = Solo<N1, N2>;
+    extern __shared__ __align__(16) float4 smem4[];
+    float4 *ptab = smem4;
+    ulonglong2 *tile = reinterpret_cast<ulonglong2 *>(smem4 + PHASE_TAB);
+    const int tid = (int)threadIdx.x;
+    const int64_t plane = blockIdx.x;
+    float2 *g = a.psi + plane * (int64_t)N1 * N2;
+    const uint32_t *fq = a.fq + plane * (int64_t)N1 * N2;
+    const float4 *tw_row = a.tw_row2 + P::V * TW2_TABLE * N2;
+    const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
+    grid_release();
+    load_phase_tab(ptab, a.ptab);
+    grid_wait();
+    const uint64_t coef = a.pot[plane >> a.log_planes];
+    if (inv) plane2_rows_global<P, true>(tile, g, tw_row, tid);
+    else plane2_copy<P, true>(tile, g, tid);
+    __syncthreads();
+    solo_columns<P>(tile, inv, true, fwd, a.twc, fq, coef, a.dither, ptab, tid);
+    __syncthreads();
+    if (fwd) plane2_rows_global<P, false>(tile, g, tw_row, tid);
+    else plane2_copy<P, false>(tile, g, tid);
 }
 
 template <int N1, int N2, int C>
-__global__ void __launch_bounds__(PLANE_THREADS, plane_min_blocks<N1, N2, C>()) k_plane_pass(PlaneArgs a) {
-    using P = PlaneCfg<N1, N2, C>;
+__global__ void __launch_bounds__(Plane2<N1, N2, C, 1>::THREADS, plane2_min_blocks<Plane2<N1, N2, C, 1>>(512))
+    k_plane_pass(PlaneArgs a) {
+    using P = Plane2<N1, N2, C, 1>;
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
-    float2 *tile = reinterpret_cast<float2 *>(smem4 + PHASE_TAB);
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank();
+    ulonglong2 *tile = reinterpret_cast<ulonglong2 *>(smem4 + PHASE_TAB);
+    const int rank = (int)(blockIdx.x % C), tid = (int)threadIdx.x;
     const int64_t plane = blockIdx.x / C;
     uint32_t tiles[C];
 #pragma unroll
     for (int q = 0; q < C; ++q) tiles[q] = cluster_addr(tile, (uint32_t)q);
     float2 *g = a.psi + plane * (int64_t)N1 * N2 + (int64_t)rank * P::R * N2;
+    const float4 *tw_row = a.tw_row2 + P::V * TW2_TABLE * N2;
     const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
-
-    const uint32_t *fqr = a.fq + plane * (int64_t)N1 * N2;
+    const uint32_t *fq = a.fq + plane * (int64_t)N1 * N2;
     grid_release();
-    {
-        // the potential rows this CTA's exchange positions read (R / C rows in
-        // each of the C row blocks) go to L2 now, during the tile load and the
-        // inverse transforms, so the exchange's potential loads hit L2
-        // (measured: 163.2 -> 160.5 us per 256^3 pass)
-        constexpr uint32_t FQB = (uint32_t)((P::R / C) * N2 * sizeof(uint32_t));
-        if (FQB % 16 == 0 && (int)threadIdx.x < C) {
-            const uint32_t *src = fqr + (int64_t)(P::R * threadIdx.x + rank * (P::R / C)) * N2;
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(FQB) : "memory");
-        }
-    }
-    grid_wait();
-    plane_copy<N1, N2, C, true>(tile, g);
     load_phase_tab(ptab, a.ptab);
-    const uint64_t coef = a.pot[plane / a.planes_per_inst];
-    plane_copy_wait();
+    grid_wait();
+    const uint64_t coef = a.pot[plane >> a.log_planes];
     if (inv) {
-        plane_rows<N1, N2, C, 1>(tile, a.tw_row, nullptr, nullptr, rank);
+        plane2_rows_global<P, true>(tile, g, tw_row, tid);
         __syncthreads();
-        plane_columns<N1, N2, C, true>(tile);
+        plane2_columns<P, true>(tile, tid);
+    } else {
+        plane2_copy<P, true>(tile, g, tid);
     }
-    cluster.sync();
-    plane_exchange<N1, N2, C, (C >= 8 ? 1 : 2)>(tiles, rank, inv, true, fwd, a.twx, fqr, coef, a.dither, ptab);
-    cluster.sync();
+    cluster_sync();
+    plane2_exchange<P>(tiles, rank, inv, true, fwd, a.twx, fq, coef, a.dither, ptab, tid);
+    cluster_sync();
     if (fwd) {
-        plane_columns<N1, N2, C, false>(tile);
+        plane2_columns<P, false>(tile, tid);
         __syncthreads();
-        plane_rows<N1, N2, C, 0>(tile, a.tw_row, nullptr, nullptr, rank);
-        __syncthreads();
+        plane2_rows_global<P, false>(tile, g, tw_row, tid);
+    } else {
+        plane2_copy<P, false>(tile, g, tid);
     }
-    plane_copy<N1, N2, C, false>(tile, g);
+}
+
+template <int N1, int N2>
+__global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1, N2>>()) k_solo_whole(PlaneArgs a) {
+    using P = Solo<N1, N2>;
+    extern __shared__ __align__(16) float4 smem4[];
+    float4 *ptab = smem4;
+    ulonglong2 *tile = reinterpret_cast<ulonglong2 *>(smem4 + PHASE_TAB);
+    grid_release();
+    load_phase_tab(ptab, a.ptab);
+    grid_wait();
+    solo_whole_run<P>(a, a.first + blockIdx.x, ptab, tile, (int)threadIdx.x);
 }
 
 // MINB: CTAs per SM the kernel is compiled for (2 for batches; 1 for the wide
@@ -86,13 +121,13 @@ __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(PlaneArgs a
 #pragma unroll
     for (int q = 0; q < C; ++q) tiles[q] = cluster_addr(tile, (uint32_t)q);
     grid_release();
-    plane_whole_run<N1, N2, C, 1>(a, blockIdx.x / C, rank, tiles, ptab, tile, true, cluster);
+    plane_whole_run<N1, N2, C, 1>(a, a.first + blockIdx.x / C, rank, tiles, ptab, tile, true, cluster);
 }
 
 // ---------------------------------------------------------------- launchers
 template <typename K>
-static cudaError_t launch_cluster(K kernel, bool overlap, int64_t clusters, int c, size_t smem, const PlaneArgs &a,
-                                  cudaStream_t s, bool &attr_done) {
+static cudaError_t launch_cluster(K kernel, bool overlap, int64_t clusters, int c, int threads, size_t smem,
+                                  const PlaneArgs &a, cudaStream_t s, bool &attr_done) {
     if (!attr_done) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -100,64 +135,113 @@ static cudaError_t launch_cluster(K kernel, bool overlap, int64_t clusters, int 
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * c), 1, 1);
-    cfg.blockDim = dim3(PLANE_THREADS, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)c;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // kernels follow qhd_launch.cuh's rules
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    int k = 0;
+    if (overlap) {  // the kernels follow qhd_launch.cuh's rules
+        attr[k].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[k++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (c > 1) {
+        attr[k].id = cudaLaunchAttributeClusterDimension;
+        attr[k].val.clusterDim.x = (unsigned)c;
+        attr[k].val.clusterDim.y = 1;
+        attr[k++].val.clusterDim.z = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = overlap ? 2 : 1;
+    cfg.numAttrs = (unsigned)k;
     return cudaLaunchKernelEx(&cfg, kernel, a);
-}
-
-// The shared-memory attribute is a per-device property of the kernel; it is set
-// on the first launch of each instantiation (one device per process here).
-template <int N1, int N2, int C>
-static cudaError_t plane_pass_impl(const PlaneArgs &a, cudaStream_t s) {
-    static bool attr_done = false;
-    return launch_cluster(k_plane_pass<N1, N2, C>, a.planes * N1 * N2 < OVERLAP_POINTS, a.planes, C, PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
-}
-
-template <int N1, int N2, int C, int MINB = 2>
-static cudaError_t plane_whole_impl(const PlaneArgs &a, cudaStream_t s) {
-    static bool attr_done = false;
-    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, true, a.batch, C, PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
 }
 
 // Cluster size per distributed-axis length: R = 32 rows per CTA (16 for 32).
 __host__ __device__ constexpr int plane_c(int n1) { return n1 >= 256 ? 8 : n1 >= 128 ? 4 : n1 >= 64 ? 2 : n1 >= 32 ? 2 : 0; }
+
+// The shared-memory attribute is a per-device property of the kernel; it is set
+// on the first launch of each instantiation (one device per process here).
+template <int N1, int N2>
+static cudaError_t plane_pass_impl(const PlaneArgs &a, cudaStream_t s) {
+    static bool attr_done = false;
+    const bool overlap = a.planes * N1 * N2 < OVERLAP_POINTS;
+    if constexpr (plane_solo(N1, N2)) {
+        using P = Solo<N1, N2>;
+        return launch_cluster(k_solo_pass<N1, N2>, overlap, a.planes, 1, P::THREADS, P::SMEM, a, s, attr_done);
+    } else {
+        using P = Plane2<N1, N2, plane_c(N1), 1>;
+        return launch_cluster(k_plane_pass<N1, N2, plane_c(N1)>, overlap, a.planes, plane_c(N1), P::THREADS, P::SMEM, a, s,
+                              attr_done);
+    }
+}
+
+template <int N1, int N2>
+static cudaError_t solo_whole_impl(const PlaneArgs &a, cudaStream_t s) {
+    if constexpr (plane_solo(N1, N2)) {
+        using P = Solo<N1, N2>;
+        static bool attr_done = false;
+        return launch_cluster(k_solo_whole<N1, N2>, true, a.instances, 1, P::THREADS, P::SMEM, a, s, attr_done);
+    } else {
+        return cudaErrorInvalidValue;
+    }
+}
+
+template <int N1, int N2, int C = plane_c(N1), int MINB = 2>
+static cudaError_t plane_whole_impl(const PlaneArgs &a, cudaStream_t s) {
+    static bool attr_done = false;
+    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, true, a.instances, C, PLANE_THREADS, PlaneCfg<N1, N2, C>::SMEM, a, s,
+                          attr_done);
+}
 
 bool plane_supported(int n1, int n2) {
     return (n1 == 32 || n1 == 64 || n1 == 128 || n1 == 256) && (n2 == 32 || n2 == 64 || n2 == 128 || n2 == 256);
 }
 
 int plane_cluster(int n1) { return plane_c(n1); }
+bool plane_fits_solo(int n1, int n2) { return plane_supported(n1, n2) && plane_solo(n1, n2); }
+
+template <int N1, int N2> static int solo_per_sm_of() {
+    if constexpr (plane_solo(N1, N2)) return solo_min_blocks<Solo<N1, N2>>();
+    else return 0;
+}
 
 #define QHD_PLANE_DISPATCH(fn)                                                        \
     switch (n1 * 1000 + n2) {                                                         \
-    case 32032: return fn<32, 32, plane_c(32)>(a, s);                                 \
-    case 32064: return fn<32, 64, plane_c(32)>(a, s);                                 \
-    case 32128: return fn<32, 128, plane_c(32)>(a, s);                                \
-    case 32256: return fn<32, 256, plane_c(32)>(a, s);                                \
-    case 64032: return fn<64, 32, plane_c(64)>(a, s);                                 \
-    case 64064: return fn<64, 64, plane_c(64)>(a, s);                                 \
-    case 64128: return fn<64, 128, plane_c(64)>(a, s);                                \
-    case 64256: return fn<64, 256, plane_c(64)>(a, s);                                \
-    case 128032: return fn<128, 32, plane_c(128)>(a, s);                              \
-    case 128064: return fn<128, 64, plane_c(128)>(a, s);                              \
-    case 128128: return fn<128, 128, plane_c(128)>(a, s);                             \
-    case 128256: return fn<128, 256, plane_c(128)>(a, s);                             \
-    case 256032: return fn<256, 32, plane_c(256)>(a, s);                              \
-    case 256064: return fn<256, 64, plane_c(256)>(a, s);                              \
-    case 256128: return fn<256, 128, plane_c(256)>(a, s);                             \
-    case 256256: return fn<256, 256, plane_c(256)>(a, s);                             \
+    case 32032: return fn<32, 32>(a, s);    \
+    case 32064: return fn<32, 64>(a, s);    \
+    case 32128: return fn<32, 128>(a, s);    \
+    case 32256: return fn<32, 256>(a, s);    \
+    case 64032: return fn<64, 32>(a, s);    \
+    case 64064: return fn<64, 64>(a, s);    \
+    case 64128: return fn<64, 128>(a, s);    \
+    case 64256: return fn<64, 256>(a, s);    \
+    case 128032: return fn<128, 32>(a, s);    \
+    case 128064: return fn<128, 64>(a, s);    \
+    case 128128: return fn<128, 128>(a, s);    \
+    case 128256: return fn<128, 256>(a, s);    \
+    case 256032: return fn<256, 32>(a, s);    \
+    case 256064: return fn<256, 64>(a, s);    \
+    case 256128: return fn<256, 128>(a, s);    \
+    case 256256: return fn<256, 256>(a, s);    \
     default: return cudaErrorInvalidValue;                                            \
     }
+
+int solo_per_sm(int n1, int n2) {
+    switch (n1 * 1000 + n2) {
+    case 32032: return solo_per_sm_of<32, 32>();
+    case 32064: return solo_per_sm_of<32, 64>();
+    case 32128: return solo_per_sm_of<32, 128>();
+    case 32256: return solo_per_sm_of<32, 256>();
+    case 64032: return solo_per_sm_of<64, 32>();
+    case 64064: return solo_per_sm_of<64, 64>();
+    case 64128: return solo_per_sm_of<64, 128>();
+    case 64256: return solo_per_sm_of<64, 256>();
+    case 128032: return solo_per_sm_of<128, 32>();
+    case 128064: return solo_per_sm_of<128, 64>();
+    case 128128: return solo_per_sm_of<128, 128>();
+    case 128256: return solo_per_sm_of<128, 256>();
+    default: return 0;
+    }
+}
 
 cudaError_t launch_plane_pass(int n1, int n2, const PlaneArgs &a, cudaStream_t s) {
     QHD_PLANE_DISPATCH(plane_pass_impl)
@@ -165,6 +249,10 @@ cudaError_t launch_plane_pass(int n1, int n2, const PlaneArgs &a, cudaStream_t s
 
 cudaError_t launch_plane_whole(int n1, int n2, const PlaneArgs &a, cudaStream_t s) {
     QHD_PLANE_DISPATCH(plane_whole_impl)
+}
+
+cudaError_t launch_solo_whole(int n1, int n2, const PlaneArgs &a, cudaStream_t s) {
+    QHD_PLANE_DISPATCH(solo_whole_impl)
 }
 
 // The whole-run kernel with twice the CTAs per instance (half the rows each) for
@@ -185,6 +273,54 @@ cudaError_t launch_plane_whole_wide(int n1, int n2, const PlaneArgs &a, cudaStre
     case 128128: return plane_whole_impl<128, 128, plane_c_wide(128), 1>(a, s);
     case 128256: return plane_whole_impl<128, 256, plane_c_wide(128), 1>(a, s);
     default: return cudaErrorInvalidValue;
+    }
+}
+
+// exp(-2 pi i m / n) as (re, im) values and their FP32 residuals
+static void unit_root(int64_t m, int64_t n, float *hr, float *hi, float *lr, float *li) {
+    const double ang = 2.0 * 3.141592653589793238462643383279502884 * (double)(m % n) / (double)n;
+    const double cr = cos(ang), ci = -sin(ang);
+    *hr = (float)cr;
+    *hi = (float)ci;
+    *lr = (float)(cr - (double)*hr);
+    *li = (float)(ci - (double)*hi);
+}
+
+void exchange_twiddles(float4 *out, int n1, int c) {
+    const int r = n1 / c;
+    for (int q = 0; q < c; ++q)
+        for (int j = 0; j < r; ++j) {
+            float4 &o = out[q * r + j];
+            unit_root((int64_t)j * q, n1, &o.x, &o.y, &o.z, &o.w);
+        }
+}
+
+void exchange_twiddles2(float4 *out, int n1, int c) {
+    const int rp = n1 / c / 2;
+    for (int q = 0; q < c; ++q)
+        for (int p = 0; p < rp; ++p) {
+            float4 &h = out[q * rp + p], &l = out[n1 / 2 + q * rp + p];
+            unit_root((int64_t)(2 * p) * q, n1, &h.x, &h.z, &l.x, &l.z);
+            unit_root((int64_t)(2 * p + 1) * q, n1, &h.y, &h.w, &l.y, &l.w);
+        }
+}
+
+template <int RP> static void solo_fill(float4 *out) {
+    using L = Line2<RP, 2>;
+    constexpr int R1 = L::P::R[0], R2 = L::P::R[1];
+    static_assert(L::STAGES == 2 && R1 * R2 == RP, "two stages");
+    for (int k = 0; k < RP; ++k) unit_root(k, 2 * RP, &out[k].x, &out[k].y, &out[k].z, &out[k].w);
+    for (int i = 0; i < RP; ++i) {
+        float4 &o = out[RP + i];
+        unit_root((int64_t)(i % R1) * (i / R1), RP, &o.x, &o.y, &o.z, &o.w);
+    }
+}
+
+void solo_twiddles(float4 *out, int n1) {
+    switch (n1) {
+    case 32: return solo_fill<16>(out);
+    case 64: return solo_fill<32>(out);
+    case 128: return solo_fill<64>(out);
     }
 }
 

@@ -16,6 +16,11 @@
 // thread owns each position cluster-wide, so the inverse step, the potential
 // phase (diagonal in position space) and the forward step are fused with no
 // barrier between them: two cluster barriers per Strang step.
+//
+// This is the engine of 2-D instances that do not fit one CTA (256-point axes)
+// and of small batches, where the length of the chain of one step counts and not
+// the throughput: scalar lines have the shorter one (one 128^2 instance on 8
+// CTAs 4.5 us per step, 6.0 us with packed pairs as in qhd_plane2.cuh).
 #pragma once
 #include <cooperative_groups.h>
 #include <type_traits>
@@ -87,14 +92,14 @@ __device__ __forceinline__ void plane_columns(float2 *tile) {
     }
 }
 
-// Row transforms along N2.  KIN: forward, kinetic phase, inverse (2-D whole
-// run); otherwise one direction.  The row's own storage is the exchange buffer
-// of the line engine (its content is in registers at that point).
+// Row transforms along N2: forward, kinetic phase, inverse.  The row's own
+// storage is the exchange buffer of the line engine (its content is in registers
+// at that point).
 struct WarpSyncP {
     __device__ __forceinline__ void operator()() const { __syncwarp(); }
 };
 
-template <int N1, int N2, int C, int DIR>  // DIR: 0 forward, 1 inverse, 2 forward-kinetic-inverse
+template <int N1, int N2, int C>
 __device__ __forceinline__ void plane_rows(float2 *tile, const float4 *__restrict__ tw_row, const float4 *kt0,
                                            const float4 *kt1, int rank) {
     using P = PlaneCfg<N1, N2, C>;
@@ -106,7 +111,7 @@ __device__ __forceinline__ void plane_rows(float2 *tile, const float4 *__restric
     // (lanes 0..T2-1 of warp 0, the ones that transform it below) take the mean
     // out of the shared-memory row before the row loop and add the mean's part
     // back after it, so the loop itself is the same for every row.
-    const bool zrow = DIR == 2 && rank == 0 && (int)threadIdx.x < T2;
+    const bool zrow = rank == 0 && (int)threadIdx.x < T2;
     float2 mean_part = make_float2(0.f, 0.f);
     if (zrow) {
         float2 v[E2];
@@ -129,24 +134,18 @@ __device__ __forceinline__ void plane_rows(float2 *tile, const float4 *__restric
 #pragma unroll
             for (int e = 0; e < E2; ++e) x[e] = rp[t + T2 * e];
             __syncwarp();
-            if (DIR == 1) {
-                line_fft<N2, true>(x, rp, t, tw_row, WarpSyncP{});
-            } else {
-                line_fft<N2, false>(x, rp, t, tw_row, WarpSyncP{});
-                if (DIR == 2) {
-                    // this local row holds frequency rank + C * row along the distributed axis
-                    // plain (coherent) loads: the batched persistent kernel writes
-                    // these tables earlier in the same launch
-                    const float4 k0 = kt0[rank + C * row];
+            line_fft<N2, false>(x, rp, t, tw_row, WarpSyncP{});
+            // this local row holds frequency rank + C * row along the distributed axis
+            // plain (coherent) loads: the batched persistent kernel writes
+            // these tables earlier in the same launch
+            const float4 k0 = kt0[rank + C * row];
 #pragma unroll
-                    for (int e = 0; e < E2; ++e) {
-                        const float4 k1 = kt1[t + T2 * e];
-                        float2 y = cmul_comp(x[e], make_float2(k0.x, k0.y), make_float2(k0.z, k0.w));
-                        x[e] = cmul_comp(y, make_float2(k1.x, k1.y), make_float2(k1.z, k1.w));
-                    }
-                    line_fft<N2, true>(x, rp, t, tw_row, WarpSyncP{});
-                }
+            for (int e = 0; e < E2; ++e) {
+                const float4 k1 = kt1[t + T2 * e];
+                float2 y = cmul_comp(x[e], make_float2(k0.x, k0.y), make_float2(k0.z, k0.w));
+                x[e] = cmul_comp(y, make_float2(k1.x, k1.y), make_float2(k1.z, k1.w));
             }
+            line_fft<N2, true>(x, rp, t, tw_row, WarpSyncP{});
 #pragma unroll
             for (int e = 0; e < E2; ++e) rp[t + T2 * e] = x[e];
         }
@@ -282,7 +281,7 @@ __device__ __forceinline__ void plane_whole_run(const PlaneArgs &a, int64_t b, i
         plane_columns<N1, N2, C, false>(tile);
         __syncthreads();
         const float4 *kb = a.kt + ((int64_t)j * a.kt_batch + (a.kt_batch == 1 ? 0 : b)) * a.ksum;
-        plane_rows<N1, N2, C, 2>(tile, a.tw_row, kb, kb + N1, rank);
+        plane_rows<N1, N2, C>(tile, a.tw_row, kb, kb + N1, rank);
         __syncthreads();
         plane_columns<N1, N2, C, true>(tile);
         cluster.sync();
