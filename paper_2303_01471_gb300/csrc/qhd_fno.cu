@@ -108,7 +108,7 @@ __global__ void k_fno_lift(const double *f, const float *sigma, const double2 *s
         q[1] = sigma[b];
         q[2] = (float)(g / d.n) / (float)d.n;
         q[3] = (float)(g % d.n) / (float)d.n;
-        *reinterpret_cast<float4 *>(&feat[p * 4]) = make_float4(q[0], q[1], q[2], q[3]);
+        if (feat) *reinterpret_cast<float4 *>(&feat[p * 4]) = make_float4(q[0], q[1], q[2], q[3]);
         if (sizeof(T) == 2 && d.C == 32) {
             // BF16 at width 32: the point's 64 bytes as four 16-byte stores
             uint32_t w[16];
@@ -263,7 +263,7 @@ __global__ void k_fno_layer_out(const float2 *S, const T *v, const float *Ww, co
         for (int c = 0; c < C; ++c) a = fmaf(W[c * C + co], row[y * C + c], a);
         const int64_t idx = bx * (int64_t)n * C + o;
         if (act) {
-            stv(&a_out[idx], a);
+            if (a_out) stv(&a_out[idx], a);
             stv(&v_out[idx], gelu(a));
         } else {
             stv(&v_out[idx], a);
@@ -380,30 +380,70 @@ __global__ void __launch_bounds__(FT) k_fno_frags(uint4 *dfty, uint4 *lay, uint4
     }
 }
 
+// Axis-1 truncated DFT stage of row bx from its bf16 pairs Vt[c][y pair] in shared
+// memory: each warp owns one 16 x 8 tile of D (k_fno_dfty_tc), the scaled result
+// goes out through Ds.  Called by the whole block.
+__device__ __forceinline__ void dfty_tile(const uint32_t *Vt, float *Ds, const Dims &d, int64_t bx, float s0, float s1,
+                                          float2 *out, const uint4 *fr) {
+    const int n = d.n, M = d.M, LDV = n / 2 + 4;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int r = lane / 4, q = 2 * (lane % 4);
+    const int mt = warp / 4, nt = warp % 4;  // 2 x 4 tiles of 16 x 8
+    float acc[4] = {};
+    const int ka = 16 * mt + r, kb = ka + 8, c = 8 * nt + r;
+    const uint4 *frm = fr + (size_t)mt * (n / 16) * 32 + lane;
+    for (int y0 = 0; y0 < n; y0 += 16) {
+        const int y = y0 + q;
+        const uint4 A = __ldg(&frm[(y0 / 16) * 32]);
+        mma_bf16(acc, A.x, A.y, A.z, A.w, Vt[c * LDV + y / 2], Vt[c * LDV + y / 2 + 4]);
+    }
+    const int co = 8 * nt + q;
+    Ds[ka * 33 + co] = acc[0];
+    Ds[ka * 33 + co + 1] = acc[1];
+    Ds[kb * 33 + co] = acc[2];
+    Ds[kb * 33 + co + 1] = acc[3];
+    __syncthreads();
+    for (int o = threadIdx.x; o < M * TC_C; o += blockDim.x) {
+        const int ky = o / TC_C, cc = o % TC_C;
+        const float sc = ky == 0 ? s0 : s1;
+        out[bx * (int64_t)M * TC_C + o] = make_float2(Ds[ky * 33 + cc] * sc, Ds[(16 + ky) * 33 + cc] * sc);
+    }
+}
+
 // Layer output of row bx = (b, x) on the tensor cores:
 //   a[y][o] = sum_c v[y][c] Ww[o][c] + sum_k T[y][k] U[k][o] + bw[o],
 //   T[y][k] = cos(2 pi k y / n) (k < 16), -sin(2 pi (k - 16) y / n) (k >= 16),
 //   U[k][o] = c_k Re S[k][o] / n^2, U[16 + k][o] = c_k Im S[k][o] / n^2 (zero for k >= M),
 // which is n^-2 sum_ky c_ky Re(S[ky] e^{+2 pi i ky y / n}) as in k_fno_layer_out.
 // Each warp takes 16 rows y at a time: K = 32 (channels) + 32 (spectral).
+// The columns of B are stored in an order that gives each lane eight neighbouring
+// channels of its rows, one 16-byte store each (4-byte stores before).  a_out
+// (the pre-activation, which only the backward pass reads) may be null.
+// 128^2 x 512, per layer: 494 us with 4-byte stores and a_out, 421 us without.
 __global__ void __launch_bounds__(FT) k_fno_layer_out_tc(const float2 *S, const __nv_bfloat16 *v, const float *Ww,
                                                          const float *bw, Dims d, int act, __nv_bfloat16 *a_out,
                                                          __nv_bfloat16 *v_out, const uint4 *lay) {
-    __shared__ uint32_t Wb[TC_C * TC_LD], Ub[TC_C * TC_LD];  // [o][k pair]
+    __shared__ uint32_t Wb[TC_C * TC_LD], Ub[TC_C * TC_LD];  // [column][k pair]
     __shared__ float bs[TC_C];
     const int n = d.n, M = d.M;
     const int64_t bx = blockIdx.x;
     const float inv = 1.f / ((float)n * (float)n);
+    // column 8 nt + i of B is channel 8 (i / 2) + 2 nt + i % 2
+    auto channel = [](int col) { return 8 * ((col % 8) / 2) + 2 * (col / 8) + col % 2; };
     for (int i = threadIdx.x; i < TC_C * 16; i += blockDim.x) {
         const int o = i / 16, j = i % 16;
-        Wb[o * TC_LD + j] = bf2(Ww[o * TC_C + 2 * j], Ww[o * TC_C + 2 * j + 1]);
+        const float2 w = *reinterpret_cast<const float2 *>(&Ww[channel(o) * TC_C + 2 * j]);
+        Wb[o * TC_LD + j] = bf2(w.x, w.y);
+    }
+    for (int i = threadIdx.x; i < TC_C * 16; i += blockDim.x) {
+        const int o = i % TC_C, j = i / TC_C, ch = channel(o);
         // spectral rows 2j, 2j + 1 of U (k < 16: real parts, k >= 16: imaginary parts)
         float u[2];
         for (int e = 0; e < 2; ++e) {
             const int k = 2 * j + e, ky = k & 15;
             float val = 0.f;
             if (ky < M) {
-                const float2 sv = S[(bx * M + ky) * (int64_t)TC_C + o];
+                const float2 sv = S[(bx * M + ky) * (int64_t)TC_C + ch];
                 val = (ky == 0 ? 1.f : 2.f) * inv * (k < 16 ? sv.x : sv.y);
             }
             u[e] = val;
@@ -413,7 +453,7 @@ __global__ void __launch_bounds__(FT) k_fno_layer_out_tc(const float2 *S, const 
     for (int i = threadIdx.x; i < TC_C; i += blockDim.x) bs[i] = bw[i];
     __syncthreads();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int r = lane / 4, q = 2 * (lane % 4);
+    const int r = lane / 4, ql = lane % 4, q = 2 * ql;
     const uint32_t *vrow = reinterpret_cast<const uint32_t *>(v + bx * (int64_t)n * TC_C);
     for (int y0 = 16 * warp; y0 < n; y0 += 16 * (FT / 32)) {
         float acc[4][4] = {};
@@ -440,21 +480,21 @@ __global__ void __launch_bounds__(FT) k_fno_layer_out_tc(const float2 *S, const 
                 mma_bf16(acc[nt], A.x, A.y, A.z, A.w, Ub[o * TC_LD + k / 2], Ub[o * TC_LD + k / 2 + 4]);
             }
         }
+        // this lane's channels 8 ql + 2 nt, + 1 of rows y0 + r and y0 + r + 8
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int o = 8 * nt + q;
+        for (int h = 0; h < 2; ++h) {
+            const int y = y0 + r + 8 * h;
+            const int64_t idx = (bx * (int64_t)n + y) * TC_C + 8 * ql;
+            uint32_t w[4], pre[4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int y = y0 + r + 8 * h;
+            for (int nt = 0; nt < 4; ++nt) {
+                const int o = 8 * ql + 2 * nt;
                 const float x0 = acc[nt][2 * h] + bs[o], x1 = acc[nt][2 * h + 1] + bs[o + 1];
-                const int64_t idx = (bx * (int64_t)n + y) * TC_C + o;
-                if (act) {
-                    *reinterpret_cast<uint32_t *>(&a_out[idx]) = bf2(x0, x1);
-                    *reinterpret_cast<uint32_t *>(&v_out[idx]) = bf2(gelu(x0), gelu(x1));
-                } else {
-                    *reinterpret_cast<uint32_t *>(&v_out[idx]) = bf2(x0, x1);
-                }
+                pre[nt] = bf2(x0, x1);
+                w[nt] = act ? bf2(gelu(x0), gelu(x1)) : pre[nt];
             }
+            if (act && a_out) *reinterpret_cast<uint4 *>(&a_out[idx]) = make_uint4(pre[0], pre[1], pre[2], pre[3]);
+            *reinterpret_cast<uint4 *>(&v_out[idx]) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
 }
@@ -525,36 +565,36 @@ __global__ void __launch_bounds__(FT) k_fno_dfty_tc(const T *in, Dims d, float s
                                                     const uint4 *fr) {
     __shared__ uint32_t Vt[TC_C * (128 + 4)];  // [c][y pair], n <= 256
     __shared__ float Ds[32 * 33];
-    const int n = d.n, M = d.M, LDV = n / 2 + 4;
+    const int n = d.n, LDV = n / 2 + 4;
     const int64_t bx = blockIdx.x;
     const T *src = in + bx * (int64_t)n * TC_C;
-    for (int i = threadIdx.x; i < TC_C * (n / 2); i += blockDim.x) {
-        const int c = i % TC_C, j = i / TC_C;
-        Vt[c * LDV + j] = bf2(ldv(&src[(2 * j) * TC_C + c]), ldv(&src[(2 * j + 1) * TC_C + c]));
+    if constexpr (sizeof(T) == 2) {
+        // 16 bytes (8 channels) of rows 2j and 2j + 1 per thread; four threads cover
+        // a row.  The stores of a thread start at another channel for each of the
+        // four, which puts a warp's 32 words in 32 banks.
+        for (int i = threadIdx.x; i < 4 * (n / 2); i += blockDim.x) {
+            const int g = i % 4, j = i / 4;
+            const uint4 u = *reinterpret_cast<const uint4 *>(&src[(2 * j) * TC_C + 8 * g]);
+            const uint4 w = *reinterpret_cast<const uint4 *>(&src[(2 * j + 1) * TC_C + 8 * g]);
+            uint32_t p[8] = {__byte_perm(u.x, w.x, 0x5410), __byte_perm(u.x, w.x, 0x7632), __byte_perm(u.y, w.y, 0x5410),
+                             __byte_perm(u.y, w.y, 0x7632), __byte_perm(u.z, w.z, 0x5410), __byte_perm(u.z, w.z, 0x7632),
+                             __byte_perm(u.w, w.w, 0x5410), __byte_perm(u.w, w.w, 0x7632)};
+            uint32_t t[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) t[k] = g & 1 ? p[(k + 2) % 8] : p[k];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) p[k] = g & 2 ? t[(k + 4) % 8] : t[k];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) Vt[(8 * g + (k + 2 * g) % 8) * LDV + j] = p[k];
+        }
+    } else {
+        for (int i = threadIdx.x; i < TC_C * (n / 2); i += blockDim.x) {
+            const int c = i % TC_C, j = i / TC_C;
+            Vt[c * LDV + j] = bf2(ldv(&src[(2 * j) * TC_C + c]), ldv(&src[(2 * j + 1) * TC_C + c]));
+        }
     }
     __syncthreads();
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int r = lane / 4, q = 2 * (lane % 4);
-    const int mt = warp / 4, nt = warp % 4;  // 2 x 4 tiles of 16 x 8
-    float acc[4] = {};
-    const int ka = 16 * mt + r, kb = ka + 8, c = 8 * nt + r;
-    const uint4 *frm = fr + (size_t)mt * (n / 16) * 32 + lane;
-    for (int y0 = 0; y0 < n; y0 += 16) {
-        const int y = y0 + q;
-        const uint4 A = __ldg(&frm[(y0 / 16) * 32]);
-        mma_bf16(acc, A.x, A.y, A.z, A.w, Vt[c * LDV + y / 2], Vt[c * LDV + y / 2 + 4]);
-    }
-    const int co = 8 * nt + q;
-    Ds[ka * 33 + co] = acc[0];
-    Ds[ka * 33 + co + 1] = acc[1];
-    Ds[kb * 33 + co] = acc[2];
-    Ds[kb * 33 + co + 1] = acc[3];
-    __syncthreads();
-    for (int o = threadIdx.x; o < M * TC_C; o += blockDim.x) {
-        const int ky = o / TC_C, cc = o % TC_C;
-        const float sc = ky == 0 ? s0 : s1;
-        out[bx * (int64_t)M * TC_C + o] = make_float2(Ds[ky * 33 + cc] * sc, Ds[(16 + ky) * 33 + cc] * sc);
-    }
+    dfty_tile(Vt, Ds, d, bx, s0, s1, out, fr);
 }
 
 // Backward of the layer input on the tensor cores (BF16 path), as k_fno_layer_in_bwd:
@@ -728,89 +768,116 @@ __global__ void __launch_bounds__(FT) k_fno_proj_bwd_tc(const __nv_bfloat16 *v, 
 // X and Y2 enter the products as BF16, transposed into shared memory; each
 // warp computes the real and the imaginary tile of the same rows, so it writes
 // complex outputs directly.
-template <bool ADJ>
+// NB instances per block share the loads of the mode weights (256 KB per ky and
+// block, from L2): 128^2 x 512, 340 us per layer with one instance per block, 310
+// with four.  The adjoint reads a mode's weights along its rows and passes them
+// through shared memory (64 instances: 172 us per layer with the strided reads, 103).
+template <bool ADJ, int NB>
 __global__ void __launch_bounds__(FT) k_fno_specx_tc(const float2 *in, const float2 *R, Dims d, float2 *mid,
                                                      float2 *out, const uint4 *sx1, const uint4 *sx2) {
     extern __shared__ __align__(16) uint32_t sm32[];
     const int n = d.n, M = d.M, MX = d.MX;
     const int LDX = n + 4;                         // words per row of Xt: n/2 (re) pairs, n/2 (im) pairs, padding
-    uint32_t *Xt = sm32;                           // [c][k pair], k over (re x | im x), 2n values
-    float2 *Y1 = reinterpret_cast<float2 *>(Xt + TC_C * LDX);  // [kx][c]
-    float2 *Y2 = Y1 + MX * TC_C;                   // [kx][c]
-    uint32_t *Yt = reinterpret_cast<uint32_t *>(Y2 + MX * TC_C);  // [c][k pair], k over (re kx | im kx), 2 MX values
     constexpr int LDY = 32 + 4;
-    const int64_t b = blockIdx.x / M;
-    const int ky = blockIdx.x - (int)(b * M);
-    for (int i = threadIdx.x; i < TC_C * (n / 2); i += blockDim.x) {
-        const int c = i % TC_C, j = i / TC_C;  // x pair (2j, 2j + 1)
-        const float2 v0 = in[((b * n + 2 * j) * M + ky) * (int64_t)TC_C + c];
-        const float2 v1 = in[((b * n + 2 * j + 1) * M + ky) * (int64_t)TC_C + c];
-        Xt[c * LDX + j] = bf2(v0.x, v1.x);
-        Xt[c * LDX + n / 2 + j] = bf2(v0.y, v1.y);
-    }
-    __syncthreads();
+    uint32_t *Xt = sm32;                           // [c][k pair], k over (re x | im x), 2n values
+    float2 *Y1 = reinterpret_cast<float2 *>(Xt + TC_C * LDX);             // [instance][kx][c]
+    uint32_t *Yt = reinterpret_cast<uint32_t *>(Y1 + NB * MX * TC_C);     // [instance][c][k pair], k over (re kx | im kx)
+    float2 *Rs = reinterpret_cast<float2 *>(Yt + NB * TC_C * LDY);        // adjoint: a mode's weights per warp
+    const int64_t g = blockIdx.x / M;
+    const int ky = blockIdx.x - (int)(g * M);
+    const int64_t b0 = g * NB;
+    const int nb = d.B - b0 < NB ? (int)(d.B - b0) : NB;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int r = lane / 4, q = 2 * (lane % 4);
     const int S1 = 2 * n / 16, S2 = 2 * MX / 16;
     // ---- Y1: warp -> (kx tile kt, column tile nt); real and imaginary rows together
-    for (int t = warp; t < (MX / 16) * 4; t += FT / 32) {
-        const int kt = t / 4, nt = t % 4;
-        const int ka = 16 * kt + r, kb = ka + 8;
-        float re[4] = {}, im[4] = {};
-        const int c = 8 * nt + r;
-        for (int k0 = 0; k0 < 2 * n; k0 += 16) {
-            // real rows: cos . Re X + sin . Im X;  imaginary rows: -sin . Re X + cos . Im X
-            const uint4 *fa = &sx1[(((size_t)kt * S1 + k0 / 16) * 2) * 32 + lane];
-            const uint4 A = __ldg(fa), B = __ldg(fa + 32);
-            const uint32_t ar[4] = {A.x, A.y, A.z, A.w}, ai[4] = {B.x, B.y, B.z, B.w};
-            const int kw = (k0 + q) / 2;
-            const uint32_t b0 = Xt[c * LDX + kw], b1 = Xt[c * LDX + kw + 4];
-            mma_bf16(re, ar[0], ar[1], ar[2], ar[3], b0, b1);
-            mma_bf16(im, ai[0], ai[1], ai[2], ai[3], b0, b1);
+    for (int i0 = 0; i0 < nb; ++i0) {
+        const int64_t b = b0 + i0;
+        if (i0) __syncthreads();
+        for (int i = threadIdx.x; i < TC_C * (n / 2); i += blockDim.x) {
+            const int c = i % TC_C, j = i / TC_C;  // x pair (2j, 2j + 1)
+            const float2 v0 = in[((b * n + 2 * j) * M + ky) * (int64_t)TC_C + c];
+            const float2 v1 = in[((b * n + 2 * j + 1) * M + ky) * (int64_t)TC_C + c];
+            Xt[c * LDX + j] = bf2(v0.x, v1.x);
+            Xt[c * LDX + n / 2 + j] = bf2(v0.y, v1.y);
         }
-        const int co = 8 * nt + q;
-        const float2 ya0 = make_float2(re[0], im[0]), ya1 = make_float2(re[1], im[1]);
-        const float2 yb0 = make_float2(re[2], im[2]), yb1 = make_float2(re[3], im[3]);
-        Y1[ka * TC_C + co] = ya0;
-        Y1[ka * TC_C + co + 1] = ya1;
-        Y1[kb * TC_C + co] = yb0;
-        Y1[kb * TC_C + co + 1] = yb1;
-        mid[((b * MX + ka) * M + ky) * (int64_t)TC_C + co] = ya0;
-        mid[((b * MX + ka) * M + ky) * (int64_t)TC_C + co + 1] = ya1;
-        mid[((b * MX + kb) * M + ky) * (int64_t)TC_C + co] = yb0;
-        mid[((b * MX + kb) * M + ky) * (int64_t)TC_C + co + 1] = yb1;
-    }
-    __syncthreads();
-    // ---- mode mixing (FP32), then Y2 as BF16 pairs over (re kx | im kx)
-    for (int o = threadIdx.x; o < MX * TC_C; o += blockDim.x) {
-        const int kx = o / TC_C, c = o - kx * TC_C;
-        const float2 *Rm = R + ((int64_t)(kx * M + ky) * TC_C) * TC_C;  // [i][o]
-        float re = 0.f, im = 0.f;
-        for (int j = 0; j < TC_C; ++j) {
-            const float2 y = Y1[kx * TC_C + j];
-            if (!ADJ) {
-                const float2 rr = Rm[j * TC_C + c];
-                re += rr.x * y.x - rr.y * y.y;
-                im += rr.x * y.y + rr.y * y.x;
-            } else {
-                const float2 rr = Rm[c * TC_C + j];
-                re += rr.x * y.x + rr.y * y.y;
-                im += rr.x * y.y - rr.y * y.x;
+        __syncthreads();
+        for (int t = warp; t < (MX / 16) * 4; t += FT / 32) {
+            const int kt = t / 4, nt = t % 4;
+            const int ka = 16 * kt + r, kb = ka + 8;
+            float re[4] = {}, im[4] = {};
+            const int c = 8 * nt + r;
+            for (int k0 = 0; k0 < 2 * n; k0 += 16) {
+                // real rows: cos . Re X + sin . Im X;  imaginary rows: -sin . Re X + cos . Im X
+                const uint4 *fa = &sx1[(((size_t)kt * S1 + k0 / 16) * 2) * 32 + lane];
+                const uint4 A = __ldg(fa), B = __ldg(fa + 32);
+                const int kw = (k0 + q) / 2;
+                const uint32_t x0 = Xt[c * LDX + kw], x1 = Xt[c * LDX + kw + 4];
+                mma_bf16(re, A.x, A.y, A.z, A.w, x0, x1);
+                mma_bf16(im, B.x, B.y, B.z, B.w, x0, x1);
+            }
+            const int co = 8 * nt + q;
+            const float4 ya = make_float4(re[0], im[0], re[1], im[1]), yb = make_float4(re[2], im[2], re[3], im[3]);
+            float2 *y = Y1 + i0 * MX * TC_C;
+            *reinterpret_cast<float4 *>(&y[ka * TC_C + co]) = ya;
+            *reinterpret_cast<float4 *>(&y[kb * TC_C + co]) = yb;
+            if (mid) {
+                *reinterpret_cast<float4 *>(&mid[((b * MX + ka) * M + ky) * (int64_t)TC_C + co]) = ya;
+                *reinterpret_cast<float4 *>(&mid[((b * MX + kb) * M + ky) * (int64_t)TC_C + co]) = yb;
             }
         }
-        Y2[o] = make_float2(re, im);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < TC_C * (MX / 2); i += blockDim.x) {
-        const int c = i % TC_C, j = i / TC_C;  // kx pair (2j, 2j + 1)
-        const float2 v0 = Y2[(2 * j) * TC_C + c], v1 = Y2[(2 * j + 1) * TC_C + c];
-        Yt[c * LDY + j] = bf2(v0.x, v1.x);
-        Yt[c * LDY + MX / 2 + j] = bf2(v0.y, v1.y);
+    // ---- mode mixing (FP32) of kx pairs (2j, 2j + 1), written as BF16 pairs over (re kx | im kx)
+    for (int o = threadIdx.x; o < (MX / 2) * TC_C; o += blockDim.x) {
+        const int j2 = o / TC_C, c = o - j2 * TC_C;
+        float2 y2[2][NB];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int kx = 2 * j2 + h;
+            const float2 *Rm = R + ((int64_t)(kx * M + ky) * TC_C) * TC_C;  // [i][o]
+            if (ADJ) {
+                // lane c needs row c: read the rows along the lanes, pass them
+                // through the warp's tile (a warp holds one j2, lanes are the channels)
+                float2 *Rt = Rs + warp * (TC_C * (TC_C + 1));
+                __syncwarp();
+#pragma unroll 8
+                for (int i = 0; i < TC_C; ++i) Rt[i * (TC_C + 1) + lane] = __ldg(&Rm[i * TC_C + lane]);
+                __syncwarp();
+            }
+            float re[NB] = {}, im[NB] = {};
+#pragma unroll 8
+            for (int j = 0; j < TC_C; ++j) {
+                const float2 rr = ADJ ? Rs[warp * (TC_C * (TC_C + 1)) + c * (TC_C + 1) + j] : Rm[j * TC_C + c];
+#pragma unroll
+                for (int i = 0; i < NB; ++i) {
+                    const float2 y = Y1[(i * MX + kx) * TC_C + j];
+                    if (!ADJ) {
+                        re[i] += rr.x * y.x - rr.y * y.y;
+                        im[i] += rr.x * y.y + rr.y * y.x;
+                    } else {
+                        re[i] += rr.x * y.x + rr.y * y.y;
+                        im[i] += rr.x * y.y - rr.y * y.x;
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < NB; ++i) y2[h][i] = make_float2(re[i], im[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            uint32_t *yt = Yt + i * TC_C * LDY + c * LDY;
+            yt[j2] = bf2(y2[0][i].x, y2[1][i].x);
+            yt[MX / 2 + j2] = bf2(y2[0][i].y, y2[1][i].y);
+        }
     }
     __syncthreads();
-    // ---- out: warp -> (x tile, column tile); real and imaginary rows together
-    for (int t = warp; t < (n / 16) * 4; t += FT / 32) {
-        const int xt = t / 4, nt = t % 4;
+    // ---- out: warp -> (instance, x tile, column tile); real and imaginary rows together
+    for (int t = warp; t < nb * (n / 16) * 4; t += FT / 32) {
+        const int i0 = t / (n / 4), t2 = t - i0 * (n / 4);
+        const int64_t b = b0 + i0;
+        const uint32_t *yt = Yt + i0 * TC_C * LDY;
+        const int xt = t2 / 4, nt = t2 % 4;
         const int xa = 16 * xt + r, xb = xa + 8;
         float re[4] = {}, im[4] = {};
         const int c = 8 * nt + r;
@@ -818,22 +885,32 @@ __global__ void __launch_bounds__(FT) k_fno_specx_tc(const float2 *in, const flo
             // real rows: cos . Re Y2 - sin . Im Y2;  imaginary rows: sin . Re Y2 + cos . Im Y2
             const uint4 *fa = &sx2[(((size_t)xt * S2 + k0 / 16) * 2) * 32 + lane];
             const uint4 A = __ldg(fa), B = __ldg(fa + 32);
-            const uint32_t ar[4] = {A.x, A.y, A.z, A.w}, ai[4] = {B.x, B.y, B.z, B.w};
             const int kw = (k0 + q) / 2;
-            const uint32_t b0 = Yt[c * LDY + kw], b1 = Yt[c * LDY + kw + 4];
-            mma_bf16(re, ar[0], ar[1], ar[2], ar[3], b0, b1);
-            mma_bf16(im, ai[0], ai[1], ai[2], ai[3], b0, b1);
+            const uint32_t x0 = yt[c * LDY + kw], x1 = yt[c * LDY + kw + 4];
+            mma_bf16(re, A.x, A.y, A.z, A.w, x0, x1);
+            mma_bf16(im, B.x, B.y, B.z, B.w, x0, x1);
         }
         const int co = 8 * nt + q;
-        out[((b * n + xa) * M + ky) * (int64_t)TC_C + co] = make_float2(re[0], im[0]);
-        out[((b * n + xa) * M + ky) * (int64_t)TC_C + co + 1] = make_float2(re[1], im[1]);
-        out[((b * n + xb) * M + ky) * (int64_t)TC_C + co] = make_float2(re[2], im[2]);
-        out[((b * n + xb) * M + ky) * (int64_t)TC_C + co + 1] = make_float2(re[3], im[3]);
+        *reinterpret_cast<float4 *>(&out[((b * n + xa) * M + ky) * (int64_t)TC_C + co]) =
+            make_float4(re[0], im[0], re[1], im[1]);
+        *reinterpret_cast<float4 *>(&out[((b * n + xb) * M + ky) * (int64_t)TC_C + co]) =
+            make_float4(re[2], im[2], re[3], im[3]);
     }
 }
 
-size_t smem_specx_tc(const Dims &d) {
-    return (size_t)TC_C * (d.n + 4) * 4 + 2 * (size_t)d.MX * TC_C * 8 + (size_t)TC_C * 36 * 4;
+template <bool ADJ, int NB> size_t smem_specx_tc(const Dims &d) {
+    return (size_t)TC_C * (d.n + 4) * 4 + (size_t)NB * (d.MX * TC_C * 8 + TC_C * 36 * 4) +
+           (ADJ ? (size_t)(FT / 32) * TC_C * (TC_C + 1) * sizeof(float2) : 0);
+}
+
+// Four instances per block while that still leaves every SM several blocks.
+template <bool ADJ>
+void specx_tc(const Dims &d, const float2 *in, const float2 *R, float2 *mid, float2 *out, const uint4 *sx1,
+              const uint4 *sx2, cudaStream_t s) {
+    if (d.B * d.M >= 4 * 152 * 4)
+        k_fno_specx_tc<ADJ, 4><<<(unsigned)((d.B + 3) / 4 * d.M), FT, smem_specx_tc<ADJ, 4>(d), s>>>(in, R, d, mid, out, sx1, sx2);
+    else
+        k_fno_specx_tc<ADJ, 1><<<(unsigned)(d.B * d.M), FT, smem_specx_tc<ADJ, 1>(d), s>>>(in, R, d, mid, out, sx1, sx2);
 }
 
 // Weight-gradient partials on the tensor cores (BF16 path, Cc = 32 columns of
@@ -842,29 +919,27 @@ size_t smem_specx_tc(const Dims &d) {
 // over the block's range of points, as k_fno_wgrad.  Each warp takes 16 points
 // at a time: A = X^T (O x 16, X rounded to BF16), B = Y (16 x 32); the warps'
 // FP32 tiles and the FP32 column sums of X meet in shared memory.
-__global__ void __launch_bounds__(FT) k_fno_wgrad_tc(const float *X, const __nv_bfloat16 *Y, int64_t P, int O,
-                                                     double *part) {
-    __shared__ float Dsum[128 * TC_C], bsum[128];
-    for (int i = threadIdx.x; i < O * TC_C; i += blockDim.x) Dsum[i] = 0.f;
-    for (int i = threadIdx.x; i < O; i += blockDim.x) bsum[i] = 0.f;
+// A block takes 16 MT of the O rows (blockIdx.y): with all 128 in one block its
+// 198 registers left one block per SM and the loads' latency uncovered (64 x 128^2:
+// 764 us for the five gradients of a pass).
+template <int MT>
+__global__ void __launch_bounds__(FT, 3) k_fno_wgrad_tc(const float *X, const __nv_bfloat16 *Y, int64_t P, int O,
+                                                        double *part) {
+    __shared__ float Dsum[16 * MT * TC_C], bsum[16 * MT];
+    for (int i = threadIdx.x; i < 16 * MT * TC_C; i += blockDim.x) Dsum[i] = 0.f;
+    for (int i = threadIdx.x; i < 16 * MT; i += blockDim.x) bsum[i] = 0.f;
     __syncthreads();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int r = lane / 4, q = 2 * (lane % 4);
+    const int o0 = 16 * MT * blockIdx.y;
     const int64_t per_blk = ((P + gridDim.x - 1) / gridDim.x + 15) / 16 * 16;
     const int64_t p0 = (int64_t)blockIdx.x * per_blk;
     const int64_t p1 = p0 + per_blk < P ? p0 + per_blk : P;
-    const int MT = O / 16;
-    float acc[8][4][4];
-    float bacc[8][2];
-#pragma unroll
-    for (int mt = 0; mt < 8; ++mt) {
-        bacc[mt][0] = bacc[mt][1] = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
-    }
+    float acc[MT][4][4] = {};
+    float bacc[MT][2] = {};
     const unsigned short *Yh = reinterpret_cast<const unsigned short *>(Y);
+    const float *Xo = X + o0;
+#pragma unroll 2
     for (int64_t t = p0 + 16 * warp; t < p1; t += 16 * (FT / 32)) {
         // B fragments: rows (points) t + q, t + q + 1 (and + 8), column c = 8 nt + r
         uint32_t b[4][2];
@@ -877,13 +952,12 @@ __global__ void __launch_bounds__(FT) k_fno_wgrad_tc(const float *X, const __nv_
             b[nt][1] = y8 | (y9 << 16);
         }
 #pragma unroll
-        for (int mt = 0; mt < 8; ++mt) {
-            if (mt >= MT) break;
+        for (int mt = 0; mt < MT; ++mt) {
             const int oa = 16 * mt + r, ob = oa + 8;
-            const float xa0 = X[(t + q) * O + oa], xa1 = X[(t + q + 1) * O + oa];
-            const float xb0 = X[(t + q) * O + ob], xb1 = X[(t + q + 1) * O + ob];
-            const float xa8 = X[(t + q + 8) * O + oa], xa9 = X[(t + q + 9) * O + oa];
-            const float xb8 = X[(t + q + 8) * O + ob], xb9 = X[(t + q + 9) * O + ob];
+            const float xa0 = Xo[(t + q) * O + oa], xa1 = Xo[(t + q + 1) * O + oa];
+            const float xb0 = Xo[(t + q) * O + ob], xb1 = Xo[(t + q + 1) * O + ob];
+            const float xa8 = Xo[(t + q + 8) * O + oa], xa9 = Xo[(t + q + 9) * O + oa];
+            const float xb8 = Xo[(t + q + 8) * O + ob], xb9 = Xo[(t + q + 9) * O + ob];
             bacc[mt][0] += (xa0 + xa1) + (xa8 + xa9);
             bacc[mt][1] += (xb0 + xb1) + (xb8 + xb9);
             const uint32_t a0 = bf2(xa0, xa1), a1 = bf2(xb0, xb1), a2 = bf2(xa8, xa9), a3 = bf2(xb8, xb9);
@@ -892,8 +966,7 @@ __global__ void __launch_bounds__(FT) k_fno_wgrad_tc(const float *X, const __nv_
         }
     }
 #pragma unroll
-    for (int mt = 0; mt < 8; ++mt) {
-        if (mt >= MT) break;
+    for (int mt = 0; mt < MT; ++mt) {
         const int oa = 16 * mt + r, ob = oa + 8;
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
@@ -915,8 +988,13 @@ __global__ void __launch_bounds__(FT) k_fno_wgrad_tc(const float *X, const __nv_
     }
     __syncthreads();
     double *dst = part + (int64_t)blockIdx.x * (O * TC_C + O);
-    for (int i = threadIdx.x; i < O * TC_C; i += blockDim.x) dst[i] = Dsum[i];
-    for (int i = threadIdx.x; i < O; i += blockDim.x) dst[O * TC_C + i] = bsum[i];
+    for (int i = threadIdx.x; i < 16 * MT * TC_C; i += blockDim.x) dst[o0 * TC_C + i] = Dsum[i];
+    for (int i = threadIdx.x; i < 16 * MT; i += blockDim.x) dst[O * TC_C + o0 + i] = bsum[i];
+}
+
+void wgrad_tc(const float *X, const __nv_bfloat16 *Y, int64_t P, int O, double *part, int nblk, cudaStream_t s) {
+    if (O % 32 == 0) k_fno_wgrad_tc<2><<<dim3(nblk, O / 32), FT, 0, s>>>(X, Y, P, O, part);
+    else k_fno_wgrad_tc<1><<<dim3(nblk, O / 16), FT, 0, s>>>(X, Y, P, O, part);
 }
 
 bool tc_wgrad_ok(const Dims &d, int O) { return d.C == TC_C && O % 16 == 0 && O <= 128; }
@@ -1109,34 +1187,82 @@ __global__ void k_fno_wgrad(const float *X, const T *Y, int64_t P, int O, int Cc
     if ((int)threadIdx.x < O) dst[nout + threadIdx.x] = bacc;
 }
 
-// out[k] = sum over blocks of part[blk][k]
-__global__ void k_fno_reduce(const double *part, int nblk, int K, float *out) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) {
+// k_fno_wgrad for the lift at width 32 (O = 32 rows, the 4 features): a warp walks
+// the block's points eight apart, lane = row, so the gradients stream at full
+// width (the general kernel kept half of its threads idle: 234 us for 64 x 128^2).
+__global__ void __launch_bounds__(FT) k_fno_wgrad_lift(const float *X, const float *feat, int64_t P, double *part) {
+    __shared__ float sh[8][5][32];
+    const int o = threadIdx.x % 32, g = threadIdx.x / 32;
+    const int64_t per_blk = (P + gridDim.x - 1) / gridDim.x;
+    const int64_t p0 = (int64_t)blockIdx.x * per_blk;
+    const int64_t p1 = p0 + per_blk < P ? p0 + per_blk : P;
+    float acc[5] = {};
+#pragma unroll 8
+    for (int64_t p = p0 + g; p < p1; p += 8) {
+        const float x = X[p * 32 + o];
+        const float4 q = *reinterpret_cast<const float4 *>(&feat[p * 4]);
+        acc[0] = fmaf(x, q.x, acc[0]);
+        acc[1] = fmaf(x, q.y, acc[1]);
+        acc[2] = fmaf(x, q.z, acc[2]);
+        acc[3] = fmaf(x, q.w, acc[3]);
+        acc[4] += x;
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) sh[g][k][o] = acc[k];
+    __syncthreads();
+    if (g < 5) {
         double s = 0;
-        for (int b = 0; b < nblk; ++b) s += part[(int64_t)b * K + k];
+        for (int i = 0; i < 8; ++i) s += sh[i][g][o];
+        part[(int64_t)blockIdx.x * 160 + (g < 4 ? o * 4 + g : 128 + o)] = s;
+    }
+}
+
+// out[k] = sum over blocks of part[blk][k]: a block of FT threads takes 32 outputs,
+// each summed by 8 threads over an eighth of the rows and then in a fixed order
+// (one thread per output summed 512 rows one after the other: 91 us, whatever K).
+__global__ void __launch_bounds__(FT) k_fno_reduce(const double *part, int nblk, int K, float *out) {
+    __shared__ double sh[FT];
+    const int k = blockIdx.x * 32 + threadIdx.x % 32, g = threadIdx.x / 32;
+    const int per = (nblk + 7) / 8, b1 = min(nblk, (g + 1) * per);
+    double s = 0;
+    if (k < K)
+#pragma unroll 8
+        for (int b = g * per; b < b1; ++b) s += part[(int64_t)b * K + k];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    if (g == 0 && k < K) {
+        for (int i = 1; i < 8; ++i) s += sh[32 * i + threadIdx.x];
         out[k] = (float)s;
     }
 }
 
 // gradient of the spectral weights: dR[kx][ky][i][o] = sum_b dW_b[kx][ky][o] conj(V_b[kx][ky][i])
-__global__ void k_fno_dR(const float2 *dW, const float2 *V, Dims d, float2 *dR) {
-    extern __shared__ float smem[];
+__global__ void __launch_bounds__(FT) k_fno_dR(const float2 *dW, const float2 *V, Dims d, float2 *dR) {
+    constexpr int BB = 16;  // instances per barrier (one at a time: 88 us for 64 instances)
+    __shared__ float2 vs[BB * 32], ws[BB * 32];
     const int C = d.C, MM = d.MX * d.M;
-    float2 *vs = reinterpret_cast<float2 *>(smem), *ws = vs + C;
     const int mode = blockIdx.x;  // kx * M + ky
     float2 acc[4] = {};
-    for (int64_t b = 0; b < d.B; ++b) {
+    int qi[4], qo[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int q = threadIdx.x + k * FT;
+        qi[k] = q < C * C ? q / C : 0;
+        qo[k] = q < C * C ? q - qi[k] * C : 0;
+    }
+    for (int64_t b0 = 0; b0 < d.B; b0 += BB) {
+        const int nb = d.B - b0 < BB ? (int)(d.B - b0) : BB;
         __syncthreads();
-        for (int i = threadIdx.x; i < C; i += blockDim.x) {
-            vs[i] = V[(b * MM + mode) * (int64_t)C + i];
-            ws[i] = dW[(b * MM + mode) * (int64_t)C + i];
+        for (int i = threadIdx.x; i < nb * C; i += blockDim.x) {
+            const int j = i / C, c = i - j * C;
+            vs[i] = V[((b0 + j) * MM + mode) * (int64_t)C + c];
+            ws[i] = dW[((b0 + j) * MM + mode) * (int64_t)C + c];
         }
         __syncthreads();
-        for (int k = 0; k < 4; ++k) {
-            const int q = threadIdx.x + k * FT;
-            if (q < C * C) {
-                const int i = q / C, o = q - i * C;
-                const float2 w = ws[o], v = vs[i];
+        for (int j = 0; j < nb; ++j) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float2 w = ws[j * C + qo[k]], v = vs[j * C + qi[k]];
                 acc[k].x += w.x * v.x + w.y * v.y;
                 acc[k].y += w.y * v.x - w.x * v.y;
             }
@@ -1386,8 +1512,10 @@ void set_smem_limits() {
     cudaFuncSetAttribute(k_fno_dfty<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     cudaFuncSetAttribute(k_fno_specx<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     cudaFuncSetAttribute(k_fno_specx<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_fno_specx_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_fno_specx_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_fno_specx_tc<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_fno_specx_tc<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_fno_specx_tc<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_fno_specx_tc<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     cudaFuncSetAttribute(k_fno_layer_out<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     cudaFuncSetAttribute(k_fno_layer_in_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
@@ -1399,31 +1527,33 @@ qhd_status forward(qhd_fno *f, const double *fx, const float *sigma, int64_t B, 
     d.B = B;
     cudaStream_t s = f->stream;
     const float *W = f->params;
+    // only a backward pass reads the features, the pre-activations and the modes
+    const bool keep = p_out == nullptr;
+    const bool tc = f->bf16 && tc_layer_ok(d);
     k_fno_fstats<<<(unsigned)B, FT, 0, s>>>(fx, d.G(), f->stats);
-    k_fno_lift<T><<<grid_for(d.P()), FT, 0, s>>>(fx, sigma, f->stats, W + f->off_lw, W + f->off_lb, d, f->feat,
-                                                 (T *)f->v[0]);
+    k_fno_lift<T><<<grid_for(d.P()), FT, 0, s>>>(fx, sigma, f->stats, W + f->off_lw, W + f->off_lb, d,
+                                                 keep ? f->feat : nullptr, (T *)f->v[0]);
     f->launches += 2;
     for (int l = 0; l < d.L; ++l) {
         const T *vin = (const T *)f->v[l];
-        if (f->bf16 && tc_layer_ok(d))
+        if (tc)
             k_fno_dfty_tc<T><<<(unsigned)(B * d.n), FT, 0, s>>>(vin, d, 1.f, 1.f, f->tspec, f->fr[0]);
         else
             k_fno_dfty<T><<<(unsigned)(B * d.n), FT, smem_dfty(d), s>>>(vin, d, 1.f, 1.f, f->tspec);
         if (f->bf16 && tc_specx_ok(d))
-            k_fno_specx_tc<false><<<(unsigned)(B * d.M), FT, smem_specx_tc(d), s>>>(
-                f->tspec, reinterpret_cast<const float2 *>(W + f->off_R[l]), d, f->vhat[l], f->sspec, f->fr[2],
-                f->fr[3]);
+            specx_tc<false>(d, f->tspec, reinterpret_cast<const float2 *>(W + f->off_R[l]),
+                            keep ? f->vhat[l] : nullptr, f->sspec, f->fr[2], f->fr[3], s);
         else
             k_fno_specx<false><<<(unsigned)(B * d.M), FT, smem_specx(d), s>>>(
                 f->tspec, reinterpret_cast<const float2 *>(W + f->off_R[l]), d, f->vhat[l], f->sspec);
         const int act = l + 1 < d.L;
-        if (f->bf16 && tc_layer_ok(d))
+        if (tc)
             k_fno_layer_out_tc<<<(unsigned)(B * d.n), FT, 0, s>>>(
                 f->sspec, (const __nv_bfloat16 *)vin, W + f->off_W[l], W + f->off_b[l], d, act,
-                act ? (__nv_bfloat16 *)f->a[l] : nullptr, (__nv_bfloat16 *)f->v[l + 1], f->fr[1]);
+                act && keep ? (__nv_bfloat16 *)f->a[l] : nullptr, (__nv_bfloat16 *)f->v[l + 1], f->fr[1]);
         else
             k_fno_layer_out<T><<<(unsigned)(B * d.n), FT, smem_layer(d), s>>>(
-                f->sspec, vin, W + f->off_W[l], W + f->off_b[l], d, act, act ? (T *)f->a[l] : nullptr,
+                f->sspec, vin, W + f->off_W[l], W + f->off_b[l], d, act, act && keep ? (T *)f->a[l] : nullptr,
                 (T *)f->v[l + 1]);
         f->launches += 3;
     }
@@ -1456,12 +1586,12 @@ qhd_status backward(qhd_fno *f, const float *p_true, int64_t B, float *grad, dou
     else
         k_fno_proj_bwd<T><<<nb, FT, sp, s>>>((const T *)f->v[d.L], f->dz, W + f->off_p1, W + f->off_p1b, W + f->off_p2,
                                               d, f->dh, f->dv, f->part);
-    k_fno_reduce<<<1, FT, 0, s>>>(f->part, nb, d.H + 1, grad + f->off_p2);
+    k_fno_reduce<<<(d.H + 1 + 31) / 32, FT, 0, s>>>(f->part, nb, d.H + 1, grad + f->off_p2);
     if (f->bf16 && tc_wgrad_ok(d, d.H))
-        k_fno_wgrad_tc<<<nb, FT, 0, s>>>(f->dh, (const __nv_bfloat16 *)f->v[d.L], P, d.H, f->part);
+        wgrad_tc(f->dh, (const __nv_bfloat16 *)f->v[d.L], P, d.H, f->part, nb, s);
     else
         k_fno_wgrad<T><<<nb, FT, 0, s>>>(f->dh, (const T *)f->v[d.L], P, d.H, d.C, f->part);
-    k_fno_reduce<<<grid_for((int64_t)d.H * d.C + d.H), FT, 0, s>>>(f->part, nb, d.H * d.C + d.H, grad + f->off_p1);
+    k_fno_reduce<<<(d.H * d.C + d.H + 31) / 32, FT, 0, s>>>(f->part, nb, d.H * d.C + d.H, grad + f->off_p1);
     f->launches += 5;
     for (int l = d.L - 1; l >= 0; --l) {
         const int act = l + 1 < d.L;
@@ -1469,10 +1599,10 @@ qhd_status backward(qhd_fno *f, const float *p_true, int64_t B, float *grad, dou
                                                         f->da);
         // pointwise weights and bias: sum over points of da (x) v_l
         if (f->bf16 && tc_wgrad_ok(d, d.C))
-            k_fno_wgrad_tc<<<nb, FT, 0, s>>>(f->da, (const __nv_bfloat16 *)f->v[l], P, d.C, f->part);
+            wgrad_tc(f->da, (const __nv_bfloat16 *)f->v[l], P, d.C, f->part, nb, s);
         else
             k_fno_wgrad<T><<<nb, FT, 0, s>>>(f->da, (const T *)f->v[l], P, d.C, d.C, f->part);
-        k_fno_reduce<<<grid_for((int64_t)d.C * d.C + d.C), FT, 0, s>>>(f->part, nb, d.C * d.C + d.C,
+        k_fno_reduce<<<(d.C * d.C + d.C + 31) / 32, FT, 0, s>>>(f->part, nb, d.C * d.C + d.C,
                                                                       grad + f->off_W[l]);
         // spectral path: adjoint of the inverse axis-1 stage, then of the axis-0 stages
         const float inv = 1.f / ((float)d.n * (float)d.n);
@@ -1481,13 +1611,12 @@ qhd_status backward(qhd_fno *f, const float *p_true, int64_t B, float *grad, dou
         else
             k_fno_dfty<float><<<(unsigned)(B * d.n), FT, smem_dfty(d), s>>>(f->da, d, inv, 2.f * inv, f->dspec);
         if (f->bf16 && tc_specx_ok(d))
-            k_fno_specx_tc<true><<<(unsigned)(B * d.M), FT, smem_specx_tc(d), s>>>(
-                f->dspec, reinterpret_cast<const float2 *>(W + f->off_R[l]), d, f->dwhat, f->tspec, f->fr[2],
-                f->fr[3]);
+            specx_tc<true>(d, f->dspec, reinterpret_cast<const float2 *>(W + f->off_R[l]), f->dwhat, f->tspec, f->fr[2],
+                           f->fr[3], s);
         else
             k_fno_specx<true><<<(unsigned)(B * d.M), FT, smem_specx(d), s>>>(
                 f->dspec, reinterpret_cast<const float2 *>(W + f->off_R[l]), d, f->dwhat, f->tspec);
-        k_fno_dR<<<(unsigned)(d.MX * d.M), FT, 2 * d.C * sizeof(float2), s>>>(
+        k_fno_dR<<<(unsigned)(d.MX * d.M), FT, 0, s>>>(
             f->dwhat, f->vhat[l], d, reinterpret_cast<float2 *>(grad + f->off_R[l]));
         if (f->bf16 && tc_layer_ok(d))
             k_fno_layer_in_bwd_tc<<<(unsigned)(B * d.n), FT, 0, s>>>(f->tspec, f->da, W + f->off_W[l], d, f->dv,
@@ -1498,8 +1627,11 @@ qhd_status backward(qhd_fno *f, const float *p_true, int64_t B, float *grad, dou
         f->launches += 7;
     }
     // lift: sum over points of dv0 (x) features
-    k_fno_wgrad<float><<<nb, FT, 0, s>>>(f->dv, f->feat, P, d.C, 4, f->part);
-    k_fno_reduce<<<grid_for(5 * d.C), FT, 0, s>>>(f->part, nb, 4 * d.C + d.C, grad + f->off_lw);
+    if (d.C == 32)
+        k_fno_wgrad_lift<<<nb, FT, 0, s>>>(f->dv, f->feat, P, f->part);
+    else
+        k_fno_wgrad<float><<<nb, FT, 0, s>>>(f->dv, f->feat, P, d.C, 4, f->part);
+    k_fno_reduce<<<(4 * d.C + d.C + 31) / 32, FT, 0, s>>>(f->part, nb, 4 * d.C + d.C, grad + f->off_lw);
     f->launches += 2;
     FNO_CHECK(f);
     if (loss_host) {
