@@ -3,6 +3,7 @@
 // Owns argument validation, the workspace layout, the per-context state and
 // the order of kernel launches of one evolve call.  Device memory and the
 // stream belong to the caller; nothing here allocates device memory.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -14,6 +15,7 @@
 #include "qhd_device.cuh"
 #include "qhd_group.h"
 #include "qhd_kernels.h"
+#include "qhd_packed.cuh"
 #include "qhd_trace.h"
 #include "qhd_sched.cuh"
 #include "qhd_spectrum.h"
@@ -107,7 +109,7 @@ Layout make_layout(int ndim, const int64_t *n, int64_t batch) {
     L.coord = take(sizeof(double) * (size_t)ksum);
     L.obs_part = take(sizeof(double) * 3 * (size_t)L.obs_blocks * (size_t)batch);
     L.obs_res = take(sizeof(double) * 3 * (size_t)batch);
-    L.mm = take(sizeof(MinMaxPart) * (size_t)L.mm_blocks * (size_t)batch);
+    L.mm = take(sizeof(MinMaxPart) * (size_t)(L.mm_blocks + 1) * (size_t)batch);  // partials, then the result
     L.total = off;
     return L;
 }
@@ -371,10 +373,22 @@ qhd_status qhd_init_grid(qhd_ctx **out, int ndim, const int64_t *n, const double
     for (int d = 0; d < ndim; ++d) {
         const size_t first = (size_t)(2 * TW2_TABLE) * (size_t)c->koff[d];
         c->tw2[d] = (float4 *)(c->work + L.tw2) + first;
+        int same = 0;  // an earlier axis of this length has the same tables
+        while (n[same] != n[d]) ++same;
+        if (same < d) {
+            const float4 *src = tw2.data() + (size_t)(2 * TW2_TABLE) * (size_t)c->koff[same];
+            std::copy(src, src + 2 * TW2_TABLE * n[d], tw2.begin() + (std::ptrdiff_t)first);
+            continue;
+        }
         for (int v = 0; v < 2; ++v) {
             int radix[4], stages = 0;
             plan2_of((int)n[d], v, radix, &stages);
             size_t at = first + (size_t)(v * TW2_TABLE) * (size_t)n[d];
+            if (v == 1 && !two_plans((int)n[d])) {  // one plan under both numbers
+                std::copy(tw2.begin() + (std::ptrdiff_t)first, tw2.begin() + (std::ptrdiff_t)at,
+                          tw2.begin() + (std::ptrdiff_t)at);
+                continue;
+            }
             int64_t l = radix[0];
             for (int st = 1; st < stages; l *= radix[st], ++st) {
                 const int64_t period = l * radix[st];
@@ -446,19 +460,16 @@ qhd_status qhd_init_grid(qhd_ctx **out, int ndim, const int64_t *n, const double
         for (int64_t j = 0; j < n[d]; ++j)
             c->coord_host[(size_t)(c->koff[d] + j)] = lo[d] + (double)j * (hi[d] - lo[d]) / (double)n[d];
 
-    cudaError_t e = cudaMemcpyAsync(c->work + L.tw, tw.data(), tw.size() * sizeof(float4),
-                                    cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->work + L.tw2, tw2.data(), tw2.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->twx, twx.data(), twx.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->twc, twc.data(), twc.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->ptab, ptab.data(), ptab.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->coord, c->coord_host.data(), c->coord_host.size() * sizeof(double),
-                            cudaMemcpyHostToDevice, c->stream);
+    // the tables lie side by side in the workspace: one upload
+    std::vector<char> tables(L.obs_part - L.tw);
+    auto stage = [&](size_t at, const void *src, size_t bytes) { memcpy(tables.data() + (at - L.tw), src, bytes); };
+    stage(L.tw, tw.data(), tw.size() * sizeof(float4));
+    stage(L.tw2, tw2.data(), tw2.size() * sizeof(float4));
+    stage(L.twx, twx.data(), twx.size() * sizeof(float4));
+    stage(L.twc, twc.data(), twc.size() * sizeof(float4));
+    stage(L.ptab, ptab.data(), ptab.size() * sizeof(float4));
+    stage(L.coord, c->coord_host.data(), c->coord_host.size() * sizeof(double));
+    cudaError_t e = cudaMemcpyAsync(c->work + L.tw, tables.data(), tables.size(), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         delete c;
@@ -473,16 +484,21 @@ static qhd_status set_potential_common(qhd_ctx *c) {
     const int64_t B = c->batch, G = c->g;
     const int nb = c->L.mm_blocks;
     QHD_LAUNCH(c, launch_minmax(c->f64, G, B, c->mm, nb, c->stream));
-    std::vector<MinMaxPart> part((size_t)(nb * B));
-    QHD_CUDA(c, cudaMemcpyAsync(part.data(), c->mm, part.size() * sizeof(MinMaxPart), cudaMemcpyDeviceToHost,
-                                c->stream));
+    // few partials are cheaper to copy than one more kernel (64^2: 44 us against 50
+    // for the call), many are not (128^2 x 512, 1 MB of them: 449 against 402)
+    const bool on_device = nb * B > 1024;
+    const MinMaxPart *from = c->mm + (on_device ? nb * B : 0);
+    if (on_device) QHD_LAUNCH(c, launch_minmax_final(c->mm, nb, B, c->mm + nb * B, c->stream));
+    const int per = on_device ? 1 : nb;
+    std::vector<MinMaxPart> part((size_t)(per * B));
+    QHD_CUDA(c, cudaMemcpyAsync(part.data(), from, part.size() * sizeof(MinMaxPart), cudaMemcpyDeviceToHost, c->stream));
     QHD_CUDA(c, cudaStreamSynchronize(c->stream));
     std::vector<InstDev> inst((size_t)B);
     for (int64_t b = 0; b < B; ++b) {
         double mn = INFINITY, mx = -INFINITY;
         int64_t am = INT64_MAX, nf = 0;
-        for (int i = 0; i < nb; ++i) {
-            const MinMaxPart &p = part[(size_t)(b * nb + i)];
+        for (int i = 0; i < per; ++i) {
+            const MinMaxPart &p = part[(size_t)(b * per + i)];
             nf += p.nonfinite;
             if (p.fmin < mn || (p.fmin == mn && p.argmin < am)) {
                 mn = p.fmin;

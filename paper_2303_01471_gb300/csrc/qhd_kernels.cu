@@ -20,6 +20,7 @@
 // turn per unit of f; the kinetic phase uses integer m^2 and a 64-bit fraction
 // of a turn per unit of m^2.  The product modulo one turn is exact to 2^-32,
 // so the FP32 sine/cosine only ever sees a reduced argument.
+#include <cmath>
 #include <type_traits>
 
 #include "qhd_device.cuh"
@@ -284,51 +285,65 @@ __global__ void k_uniform(float2 *psi, int64_t count, float v) {
         psi[i] = make_float2(v, 0.0f);
 }
 
-__global__ void k_minmax(const double *f, int64_t g, MinMaxPart *part) {
+// Lowest value (lowest index on ties), highest value and non-finite count of the
+// block's 256 threads, in thread 0.
+__device__ __forceinline__ MinMaxPart minmax_block(MinMaxPart v) {
+    __shared__ MinMaxPart sh[256];
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w /= 2) {
+        if ((int)threadIdx.x < w) {
+            const MinMaxPart o = sh[threadIdx.x + w];
+            MinMaxPart &m = sh[threadIdx.x];
+            if (o.fmin < m.fmin || (o.fmin == m.fmin && o.argmin < m.argmin)) {
+                m.fmin = o.fmin;
+                m.argmin = o.argmin;
+            }
+            m.fmax = fmax(m.fmax, o.fmax);
+            m.nonfinite += o.nonfinite;
+        }
+        __syncthreads();
+    }
+    return sh[0];
+}
+
+__global__ void __launch_bounds__(256) k_minmax(const double *f, int64_t g, MinMaxPart *part) {
     const int64_t b = blockIdx.y;
     const double *fb = f + b * g;
-    double mn = INFINITY, mx = -INFINITY;
-    int64_t am = INT64_MAX, nf = 0;
+    MinMaxPart m{INFINITY, -INFINITY, INT64_MAX, 0};
+#pragma unroll 4
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < g;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double v = fb[i];
         if (!isfinite(v)) {
-            ++nf;
+            ++m.nonfinite;
             continue;
         }
-        if (v < mn || (v == mn && i < am)) {
-            mn = v;
-            am = i;
+        if (v < m.fmin || (v == m.fmin && i < m.argmin)) {
+            m.fmin = v;
+            m.argmin = i;
         }
-        mx = fmax(mx, v);
+        m.fmax = fmax(m.fmax, v);
     }
-    __shared__ double s_mn[256], s_mx[256];
-    __shared__ int64_t s_am[256], s_nf[256];
-    s_mn[threadIdx.x] = mn;
-    s_mx[threadIdx.x] = mx;
-    s_am[threadIdx.x] = am;
-    s_nf[threadIdx.x] = nf;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w /= 2) {
-        if (threadIdx.x < w) {
-            const int o = threadIdx.x + w;
-            if (s_mn[o] < s_mn[threadIdx.x] || (s_mn[o] == s_mn[threadIdx.x] && s_am[o] < s_am[threadIdx.x])) {
-                s_mn[threadIdx.x] = s_mn[o];
-                s_am[threadIdx.x] = s_am[o];
-            }
-            s_mx[threadIdx.x] = fmax(s_mx[threadIdx.x], s_mx[o]);
-            s_nf[threadIdx.x] += s_nf[o];
+    m = minmax_block(m);
+    if (threadIdx.x == 0) part[b * gridDim.x + blockIdx.x] = m;
+}
+
+// out[b] of the nblk partials of instance b.
+__global__ void __launch_bounds__(256) k_minmax_final(const MinMaxPart *part, int nblk, MinMaxPart *out) {
+    const int64_t b = blockIdx.x;
+    MinMaxPart m{INFINITY, -INFINITY, INT64_MAX, 0};
+    for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
+        const MinMaxPart p = part[b * nblk + i];
+        if (p.fmin < m.fmin || (p.fmin == m.fmin && p.argmin < m.argmin)) {
+            m.fmin = p.fmin;
+            m.argmin = p.argmin;
         }
-        __syncthreads();
+        m.fmax = fmax(m.fmax, p.fmax);
+        m.nonfinite += p.nonfinite;
     }
-    if (threadIdx.x == 0) {
-        MinMaxPart p;
-        p.fmin = s_mn[0];
-        p.fmax = s_mx[0];
-        p.argmin = s_am[0];
-        p.nonfinite = s_nf[0];
-        part[b * gridDim.x + blockIdx.x] = p;
-    }
+    m = minmax_block(m);
+    if (threadIdx.x == 0) out[b] = m;
 }
 
 __global__ void k_quantize(const double *f, uint32_t *fq, const InstDev *inst, int64_t g, int64_t total) {
@@ -354,14 +369,26 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     return s;
 }
 
-__global__ void k_obs_partial(ObsArgs a) {
+// FP64 bounds it (5.3e11 FMA/s on the whole GPU, 1/74 of the FP32 rate), so each
+// point costs only its own products: the squared coordinate distances to x* are one table per block, and the distance is
+// compared squared, with the largest square whose root is below the radius.  With
+// a square root and the coordinates' arithmetic per point, 256^3 took 897 us.
+__global__ void __launch_bounds__(256) k_obs_partial(ObsArgs a) {
+    extern __shared__ double d2[];  // (x - x*)^2 per axis, at a.coff[d]
     const int64_t b = blockIdx.y;
     const float2 *psi = a.psi + b * a.g;
     const double *f = a.f64 + b * a.g;
     const InstDev &ip = a.inst[b];
     grid_release();
+    for (int d = 0; d < a.ndim; ++d)
+        for (int i = threadIdx.x; i < a.n[d]; i += blockDim.x) {
+            const double dx = __dsub_rn(a.coord[a.coff[d] + i], ip.xs[d]);
+            d2[a.coff[d] + i] = __dmul_rn(dx, dx);
+        }
+    __syncthreads();
     grid_wait();
     double sn = 0.0, sf = 0.0, sp = 0.0;
+#pragma unroll 4
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.g;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float2 z = psi[i];
@@ -369,17 +396,16 @@ __global__ void k_obs_partial(ObsArgs a) {
         if (a.prob) a.prob[b * a.g + i] = (float)p;
         sn += p;
         sf += p * f[i];
-        // Euclidean distance to x*, evaluated in the same operation order as a
-        // plain loop over the axes from the last to the first
-        int64_t rem = i;
-        double r2 = 0.0;
-        for (int d = a.ndim - 1; d >= 0; --d) {
-            const int idx = (int)(rem & ((1 << a.log_n[d]) - 1));
-            rem >>= a.log_n[d];
-            const double dx = __dsub_rn(a.coord[a.coff[d] + idx], ip.xs[d]);
-            r2 = __dadd_rn(r2, __dmul_rn(dx, dx));
+        // squared Euclidean distance to x*, summed in the same order as a plain
+        // loop over the axes from the last to the first
+        const uint32_t idx = (uint32_t)i;  // G <= 2^30
+        double r2 = d2[a.coff[a.ndim - 1] + (idx & (a.n[a.ndim - 1] - 1))];
+        if (a.ndim > 1) {
+            uint32_t rem = idx >> a.log_n[a.ndim - 1];
+            r2 = __dadd_rn(r2, d2[a.coff[a.ndim - 2] + (rem & (a.n[a.ndim - 2] - 1))]);
+            if (a.ndim > 2) r2 = __dadd_rn(r2, d2[rem >> a.log_n[1]]);
         }
-        if (sqrt(r2) < a.radius) sp += p;
+        if (r2 <= a.r2_max) sp += p;
     }
     __shared__ double sh[32];
     const double tn = block_sum(sn, sh);
@@ -529,9 +555,21 @@ cudaError_t launch_quantize(const double *f, uint32_t *fq, const InstDev *inst, 
 }
 
 cudaError_t launch_observables(const ObsArgs &a, int64_t batch, cudaStream_t s) {
-    cudaError_t e = launch_overlapped(true, k_obs_partial, dim3((unsigned)a.nblk, (unsigned)batch), dim3(256), 0, s, a);
+    int ksum = 0;
+    for (int d = 0; d < a.ndim; ++d) ksum += a.n[d];
+    ObsArgs o = a;
+    // squares up to this are the ones whose (correctly rounded) root is below the radius
+    o.r2_max = a.radius * a.radius;
+    while (std::sqrt(o.r2_max) < a.radius) o.r2_max = std::nextafter(o.r2_max, INFINITY);
+    while (!(std::sqrt(o.r2_max) < a.radius)) o.r2_max = std::nextafter(o.r2_max, 0.0);
+    // as many blocks as fill the GPU: the tables and the block sums cost as much as
+    // hundreds of points
+    const int64_t want = (152 * 8 + batch - 1) / batch;
+    if (want < o.nblk) o.nblk = (int)want;
+    cudaError_t e = launch_overlapped(true, k_obs_partial, dim3((unsigned)o.nblk, (unsigned)batch), dim3(256),
+                                      ksum * sizeof(double), s, o);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(true, k_obs_final, dim3((unsigned)batch), dim3(256), 0, s, a);
+    return launch_overlapped(true, k_obs_final, dim3((unsigned)batch), dim3(256), 0, s, o);
 }
 
 template <int N> static void plan2_radix(int v, int *radix, int *stages) {
@@ -547,6 +585,11 @@ void plan2_of(int n, int v, int *radix, int *stages) {
 #undef QHD_PLAN2_CASE
     default: *stages = 0;
     }
+}
+
+cudaError_t launch_minmax_final(const MinMaxPart *part, int nblk, int64_t batch, MinMaxPart *out, cudaStream_t s) {
+    k_minmax_final<<<(unsigned)batch, 256, 0, s>>>(part, nblk, out);
+    return cudaGetLastError();
 }
 
 void plan_of(int n, int *r1, int *r2) {

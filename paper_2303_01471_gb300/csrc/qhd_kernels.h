@@ -132,7 +132,8 @@ struct ObsArgs {
     int log_n[3];
     int coff[3];
     double radius;
-    int nblk;
+    double r2_max;         // set by launch_observables
+    int nblk;              // partials per instance at most
 };
 
 // Launchers; each returns the launch error (cudaSuccess on success).
@@ -143,6 +144,7 @@ cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s);
 cudaError_t launch_uniform(float2 *psi, int64_t count, float value, cudaStream_t s);
 cudaError_t launch_minmax(const double *f, int64_t g, int64_t batch, MinMaxPart *part, int nblk,
                           cudaStream_t s);
+cudaError_t launch_minmax_final(const MinMaxPart *part, int nblk, int64_t batch, MinMaxPart *out, cudaStream_t s);
 cudaError_t launch_quantize(const double *f, uint32_t *fq, const InstDev *inst, int64_t g,
                             int64_t batch, cudaStream_t s);
 cudaError_t launch_observables(const ObsArgs &a, int64_t batch, cudaStream_t s);
