@@ -12,9 +12,11 @@
 // its threads before it touches anything an earlier kernel writes, or writes
 // anything an earlier kernel reads.  grid_wait returns when the previous grid is
 // complete and its writes are visible; that grid waited for the one before it,
-// so the order is transitive.  What set_potential, set_schedule and init_grid
-// write (they synchronise the stream) may be read before it.  A launch behind an
-// ordinary kernel, copy or event keeps the ordinary stream order.
+// so the order is transitive.  Nothing that a kernel of the same stream wrote may be
+// read before it unless the host has waited for that kernel since: what is left is
+// what set_potential, set_schedule and init_grid write (they synchronise the
+// stream).  A kernel without grid_release counts as well: the wait, not the end of
+// its blocks, is what makes its writes visible.
 #pragma once
 #include <cstdint>
 

@@ -1,0 +1,52 @@
+"""Kernels whose launch overlaps the end of the kernel before (csrc/qhd_launch.cuh)
+read nothing that kernel writes before it is complete."""
+import ctypes
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import workloads
+from paper_2303_01471_gb300 import qhd
+
+REL_TOL = 1e-12   # same kernels, same block counts: identical up to FP64 rounding order
+
+
+def test_static_observables_queued_back_to_back():
+    """qhd_observables_static calls on one stream with nothing waiting in between, the
+    mesh, the box and x* changing from call to call, against the context path: each
+    call's set-up kernel writes what its reduction reads, in one array for all calls."""
+    lib = qhd.load()
+    radius = 0.3
+    configs = []
+    for seed, (shape, lo, hi) in enumerate([((64,), (0.0,), (1.0,)), ((64, 128), (-1.0, 0.0), (1.0, 2.0)),
+                                            ((8, 16, 4), (0.0, -0.5, 0.0), (1.0, 0.5, 2.0)),
+                                            ((64, 128), (0.0, 0.0), (1.0, 1.0))]):
+        d = len(shape)
+        inst = workloads.gaussian_wells(70 + seed, shape, K=4)
+        sim = qhd.QHD(shape, lo=lo, hi=hi)
+        sim.set_potential(inst.f)
+        psi = np.random.default_rng(seed).normal(size=(1, *shape, 2)).astype(np.float32)
+        sim.psi.copy_(torch.view_as_complex(torch.from_numpy(psi / np.linalg.norm(psi))).reshape(sim.psi.shape))
+        configs.append({"d": d, "n": (ctypes.c_int64 * d)(*shape), "lo": (ctypes.c_double * d)(*lo),
+                        "hi": (ctypes.c_double * d)(*hi), "psi": sim.psi.clone(), "f": torch.from_numpy(inst.f).cuda(),
+                        "ref": sim.observables(radius)[0]})
+        sim.close()
+    p = [c["ref"].p_succ for c in configs]
+    assert all(abs(p[k] - p[k - 1]) > 1e-3 for k in range(len(p)))   # another call's table would show
+    out = torch.full((200, 3), float("nan"), dtype=torch.float64, device="cuda")
+    stream = torch.cuda.current_stream()
+    torch.cuda.synchronize()
+    for call in range(out.shape[0]):
+        c = configs[call % len(configs)]
+        xs = (ctypes.c_double * 3)(*c["ref"].x_star)
+        assert lib.qhd_observables_static(c["d"], c["n"], c["lo"], c["hi"], 1, ctypes.c_void_p(c["psi"].data_ptr()),
+                                          ctypes.c_void_p(c["f"].data_ptr()), xs, radius,
+                                          ctypes.c_void_p(out[call].data_ptr()), None,
+                                          ctypes.c_void_p(stream.cuda_stream)) == qhd.QHD_OK
+    stream.synchronize()
+    for call, got in enumerate(out.cpu().numpy()):
+        ref = configs[call % len(configs)]["ref"]
+        assert got == pytest.approx(np.array([ref.norm, ref.e_f, ref.p_succ]), rel=REL_TOL, abs=1e-300), call
