@@ -158,22 +158,23 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
         // shared by every point with the same frequency index, so a plain FP32
         // rounding of it would perturb the norm coherently.  The factors of axes 1
         // and 2 are the same for the whole column: their product (hi/lo again) is
-        // formed once.
+        // formed once.  Plain loads: k_prep may still write the tables when this
+        // block starts, which the read-only path does not allow.
         const float4 *kb = a.kt + (a.kt_batch == 1 ? 0 : o) * a.ksum;
         w2 kc;
         if (a.ndim == 2) {
-            kc = w2_make(__ldg(&kb[a.koff1 + ci]), __ldg(&kb[a.koff1 + ci + 1]));
+            kc = w2_make(kb[a.koff1 + ci], kb[a.koff1 + ci + 1]);
         } else {
             int64_t i1 = ci >> a.log_n2;
             const int i2 = (int)(ci & ((1 << a.log_n2) - 1));
             if (a.perm1_c) i1 = (i1 >> a.perm1_log_r) + a.perm1_c * (i1 & ((1 << a.perm1_log_r) - 1));
-            const float4 k1 = __ldg(&kb[a.koff1 + i1]);
-            kc = w2_mul(w2_make(k1, k1), w2_make(__ldg(&kb[a.koff2 + i2]), __ldg(&kb[a.koff2 + i2 + 1])));
+            const float4 k1 = kb[a.koff1 + i1];
+            kc = w2_mul(w2_make(k1, k1), w2_make(kb[a.koff2 + i2], kb[a.koff2 + i2 + 1]));
         }
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[e] = c2_mul<false>(c2_mul_shared<false>(x[e], __ldg(&kb[t + T * e])), kc);
+        for (int e = 0; e < E; ++e) x[e] = c2_mul<false>(c2_mul_shared<false>(x[e], kb[t + T * e]), kc);
         // the mean's part: N mu = sum through the factor of frequency 0
-        if (split0 && t == 0) st_c2(slot, c2_mul<false>(c2_mul_shared<false>(ld_c2(slot), __ldg(&kb[0])), kc));
+        if (split0 && t == 0) st_c2(slot, c2_mul<false>(c2_mul_shared<false>(ld_c2(slot), kb[0]), kc));
     }
     if (a.mode & MODE_INV) line_fft2<N, V, true>(x, sm, t, tw, BlockSync{}, at);
     if (split0) {
@@ -227,13 +228,14 @@ __global__ void __launch_bounds__(ROW_THREADS) k_oned(OneDArgs a) {
         const float2 sum = line_sum_lanes<E, T>(x);
         sub_line_mean<N, E>(x, sum);
         line_fft<N, false>(x, sm, t, a.tw2, WarpSync{});
+        // plain loads, as in k_axis
         const float4 *kb = a.kt + ((int64_t)j * a.kt_batch + (a.kt_batch == 1 ? 0 : b)) * N;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const float4 k0 = __ldg(&kb[t + T * e]);
+            const float4 k0 = kb[t + T * e];
             x[e] = cmul_comp(x[e], make_float2(k0.x, k0.y), make_float2(k0.z, k0.w));
         }
-        const float4 z0 = __ldg(&kb[0]);
+        const float4 z0 = kb[0];
         const float2 mean_part = cmul_comp(sum, make_float2(z0.x, z0.y), make_float2(z0.z, z0.w));
         line_fft<N, true>(x, sm, t, a.tw2, WarpSync{});
 #pragma unroll

@@ -16,7 +16,10 @@
 // read before it unless the host has waited for that kernel since: what is left is
 // what set_potential, set_schedule and init_grid write (they synchronise the
 // stream).  A kernel without grid_release counts as well: the wait, not the end of
-// its blocks, is what makes its writes visible.
+// its blocks, is what makes its writes visible.  And nothing that an overlapped
+// kernel writes is read with __ldg or through a restrict pointer, wait or not: those
+// loads are for memory that nobody writes while the kernel is resident, and the
+// compiler may move them across the wait.
 #pragma once
 #include <cstdint>
 

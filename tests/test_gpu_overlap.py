@@ -9,6 +9,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 import workloads
+from test_gpu_parity import align_global_phase
 from paper_2303_01471_gb300 import qhd
 
 REL_TOL = 1e-12   # same kernels, same block counts: identical up to FP64 rounding order
@@ -50,3 +51,30 @@ def test_static_observables_queued_back_to_back():
     for call, got in enumerate(out.cpu().numpy()):
         ref = configs[call % len(configs)]["ref"]
         assert got == pytest.approx(np.array([ref.norm, ref.e_f, ref.p_succ]), rel=REL_TOL, abs=1e-300), call
+
+
+# 200 steps of some 40 FP32 roundings each, in two runs, add up at random: sqrt(2 * 200 * 40)
+# of half an ulp is 4e-6 of an amplitude; five times that
+ROUNDING = 2e-5
+
+
+@pytest.mark.parametrize("own_kinetic", [False, True], ids=["shared-kinetic", "own-kinetic"])
+@pytest.mark.parametrize("shape", [(64,), (1024,), (16, 16), (512, 4), (16, 16, 16), (8, 32, 32)],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_one_step_calls_match_one_call(shape, own_kinetic):
+    """Every call of one step builds its kinetic tables in the kernel before the passes
+    that read them, where the call before had its own: 200 calls queued without a
+    synchronisation against one call of 200 steps."""
+    insts = [workloads.gaussian_wells(80 + b, shape, K=4) for b in range(3)]
+    states = []
+    for calls in (1, 200):
+        sim = qhd.QHD(shape, batch=3)
+        sim.set_potential(np.stack([i.f for i in insts]))
+        sim.set_schedule([qhd.Schedule(c_phi=2.0 + (0.3 * b if own_kinetic else 0.0)) for b in range(3)])
+        sim.reset_state()
+        for _ in range(calls):
+            sim.evolve(2.0 / calls, 0.01)
+        states.append(sim.psi.cpu().numpy().astype(np.complex128))
+        sim.close()
+    for a, b in zip(*states):
+        assert np.max(np.abs(align_global_phase(b, a) - a)) <= ROUNDING * np.abs(a).max()
