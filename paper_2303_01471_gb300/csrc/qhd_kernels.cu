@@ -382,14 +382,14 @@ __global__ void __launch_bounds__(256) k_obs_partial(ObsArgs a) {
     const double *f = a.f64 + b * a.g;
     const InstDev &ip = a.inst[b];
     grid_release();
-    // the coordinates and x* too may come from the kernel before (qhd_static.cu)
-    grid_wait();
+    if (a.await_tables) grid_wait();
     for (int d = 0; d < a.ndim; ++d)
         for (int i = threadIdx.x; i < a.n[d]; i += blockDim.x) {
             const double dx = __dsub_rn(a.coord[a.coff[d] + i], ip.xs[d]);
             d2[a.coff[d] + i] = __dmul_rn(dx, dx);
         }
     __syncthreads();
+    grid_wait();
     double sn = 0.0, sf = 0.0, sp = 0.0;
 #pragma unroll 4
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.g;

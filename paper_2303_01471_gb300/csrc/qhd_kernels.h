@@ -134,6 +134,7 @@ struct ObsArgs {
     double radius;
     double r2_max;         // set by launch_observables
     int nblk;              // partials per instance at most
+    bool await_tables;     // coord and inst come from a kernel on this stream, not from a synchronised upload
 };
 
 // Launchers; each returns the launch error (cudaSuccess on success).

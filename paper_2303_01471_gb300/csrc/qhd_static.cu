@@ -154,6 +154,7 @@ extern "C" qhd_status qhd_observables_static(int ndim, const int64_t *n, const d
     }
     a.radius = radius;
     a.nblk = nblk;
+    a.await_tables = true;  // k_static_setup
     if (launch_observables(a, batch, s) != cudaSuccess) return QHD_ERR_CUDA;
     if (cudaMemcpyAsync(out_dev, scratch + S_RES_OFF, sizeof(double) * 3 * (size_t)batch,
                         cudaMemcpyDeviceToDevice, s) != cudaSuccess)
