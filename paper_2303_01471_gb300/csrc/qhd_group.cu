@@ -495,10 +495,8 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
                 pl.fq = v.fq;
                 pl.pot = v.pot;
                 pl.kt = v.kt;
-                pl.tw_row = v.tw_row;
-                pl.tw_row2 = v.tw_row2;
-                pl.twc = v.twc;
-                pl.twx = g->d_twx + (size_t)i * GROUP_TWX;
+                pl.tw_row = sub > 1 ? v.tw_row : v.tw_row2;
+                pl.twx = sub > 1 ? g->d_twx + (size_t)i * GROUP_TWX : v.twc;
                 pl.batch = v.batch;
                 pl.cnt = (int)cnt;
                 pl.final_phase = j0 + cnt == nsteps ? 1 : 0;

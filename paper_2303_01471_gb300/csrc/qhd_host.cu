@@ -762,10 +762,6 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
             w.fq = c->fq;
             w.pot = c->pot;
             w.kt = c->kt;
-            w.tw_row = c->tw[1];
-            w.tw_row2 = c->tw2[1];
-            w.twc = c->twc;
-            w.twx = c->twx;
             w.batch = B;
             w.cnt = (int)cnt;
             w.final_phase = last_chunk ? 1 : 0;
@@ -774,11 +770,21 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
             w.ptab = c->ptab;
             w.kt_batch = ktb;
             TimedScope ts(c, QHD_KCLASS_WHOLE, true);
-            w.instances = c->solo;
-            if (c->solo > 0) QHD_LAUNCH(c, launch_solo_whole((int)c->n[0], (int)c->n[1], w, c->stream));
-            w.first = c->solo;
-            w.instances = B - c->solo;
-            if (w.instances > 0) {
+            if (c->solo > 0) {
+                w.tw_row = c->tw2[1];
+                w.twx = c->twc;
+                w.count = c->solo;
+                QHD_LAUNCH(c, launch_solo_whole((int)c->n[0], (int)c->n[1], w, c->stream));
+                // the rest of the batch: the same arrays from its first instance on
+                w.psi += c->solo * c->g;
+                w.fq += c->solo * c->g;
+                w.pot += c->solo;
+                if (ktb > 1) w.kt += c->solo * c->ksum;
+            }
+            w.tw_row = c->tw[1];
+            w.twx = c->twx;
+            w.count = B - c->solo;
+            if (w.count > 0) {
                 if (c->plane_c == plane_cluster_wide((int)c->n[0]))
                     QHD_LAUNCH(c, launch_plane_whole_wide((int)c->n[0], (int)c->n[1], w, c->stream));
                 else
@@ -811,10 +817,9 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
         if (c->plane_mode == 3) {
             pl.psi = c->psi;
             pl.fq = c->fq;
-            pl.tw_row2 = c->tw2[2];
-            pl.twc = c->twc;
-            pl.twx = c->twx;
-            pl.planes = B * c->n[0];
+            pl.tw_row = c->tw2[2];
+            pl.twx = c->plane_c > 1 ? c->twx : c->twc;
+            pl.count = B * c->n[0];
             pl.log_planes = log2i(c->n[0]);
             pl.batch = B;
             pl.ptab = c->ptab;

@@ -62,29 +62,30 @@ struct AxisArgs {
                                // s / r + perm1_c * (s % r), r = 2^perm1_log_r; perm1_c = 0: natural
 };
 
-// Plane engine (qhd_plane.cu): N1 distributed over a cluster, N2 per row.
+// Plane engine (qhd_plane.cu): N1 distributed over a cluster, N2 per row.  Kept small:
+// with 152 bytes of arguments instead of 144 the compiler holds less of a step in
+// registers (one 128x64 instance: 139 of them instead of 167, 2.82 us per step instead of 2.76).
 struct PlaneArgs {
     float2 *psi;
     const uint32_t *fq;
     const uint64_t *pot;     // pass: coefficients of this pass [batch]; whole: chunk [cnt+1][batch]
     const float4 *kt;        // whole: chunk kinetic tables [cnt][batch][ksum]
-    const float4 *tw_row;    // cluster whole run: stage-2 twiddles of the row length (line_fft)
-    const float4 *tw_row2;   // others: twiddles of the row length (line_fft2), both plans
-    const float4 *twx;       // exchange twiddles: exchange_twiddles (whole), exchange_twiddles2 (pass)
-    const float4 *twc;       // solo form: column twiddles (solo_twiddles)
-    int64_t planes;          // pass: batch * n0 planes
-    int log_planes;          // pass: log2 of the planes per instance (n0)
+    const float4 *tw_row;    // row twiddles: line_fft's (cluster whole run) or line_fft2's, both plans (others)
+    const float4 *twx;       // column twiddles: exchange_twiddles (cluster whole run), exchange_twiddles2
+                             // (cluster pass), solo_twiddles (one CTA)
+    int64_t count;           // planes (pass) or instances (whole) of this launch
     int64_t batch;
-    int64_t first, instances; // whole: the instances of this launch
     int mode;                // pass: MODE_INV (previous step's inverse first), MODE_FWD
     uint32_t dither;         // pass: global phase of this step
     int cnt;                 // whole: steps in the chunk
     int final_phase;         // whole: apply pot[cnt] at the end
     int ksum;
+    int log_planes;          // pass: log2 of the planes per instance (n0)
     uint64_t dither_base;    // whole: global index of the chunk's first step
     const float4 *ptab;      // potential phase table
     int64_t kt_batch;        // whole: 1 = shared kinetic table, else batch
 };
+static_assert(sizeof(PlaneArgs) <= 144, "costs the cluster engine registers");
 
 struct OneDArgs {
     float2 *psi;

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     const int64_t plane = blockIdx.x;
     float2 *g = a.psi + plane * (int64_t)N1 * N2;
     const uint32_t *fq = a.fq + plane * (int64_t)N1 * N2;
-    const float4 *tw_row = a.tw_row2 + P::V * TW2_TABLE * N2;
+    const float4 *tw_row = a.tw_row + P::V * TW2_TABLE * N2;
     const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
     grid_release();
     load_phase_tab(ptab, a.ptab);
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     if (inv) plane2_rows_global<P, true>(tile, g, tw_row, tid);
     else plane2_copy<P, true>(tile, g, tid);
     __syncthreads();
-    solo_columns<P>(tile, inv, true, fwd, a.twc, fq, coef, a.dither, ptab, tid);
+    solo_columns<P>(tile, inv, true, fwd, a.twx, fq, coef, a.dither, ptab, tid);
     __syncthreads();
     if (fwd) plane2_rows_global<P, false>(tile, g, tw_row, tid);
     else plane2_copy<P, false>(tile, g, tid);
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(Plane2<N1, N2, C, 1>::THREADS, plane2_min_bloc
 #pragma unroll
     for (int q = 0; q < C; ++q) tiles[q] = cluster_addr(tile, (uint32_t)q);
     float2 *g = a.psi + plane * (int64_t)N1 * N2 + (int64_t)rank * P::R * N2;
-    const float4 *tw_row = a.tw_row2 + P::V * TW2_TABLE * N2;
+    const float4 *tw_row = a.tw_row + P::V * TW2_TABLE * N2;
     const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
     const uint32_t *fq = a.fq + plane * (int64_t)N1 * N2;
     grid_release();
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     grid_release();
     load_phase_tab(ptab, a.ptab);
     grid_wait();
-    solo_whole_run<P>(a, a.first + blockIdx.x, ptab, tile, (int)threadIdx.x);
+    solo_whole_run<P>(a, blockIdx.x, ptab, tile, (int)threadIdx.x);
 }
 
 // MINB: CTAs per SM the kernel is compiled for (2 for batches; 1 for the wide
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(PlaneArgs a
 #pragma unroll
     for (int q = 0; q < C; ++q) tiles[q] = cluster_addr(tile, (uint32_t)q);
     grid_release();
-    plane_whole_run<N1, N2, C, 1>(a, a.first + blockIdx.x / C, rank, tiles, ptab, tile, true, cluster);
+    plane_whole_run<N1, N2, C, 1>(a, blockIdx.x / C, rank, tiles, ptab, tile, true, cluster);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -163,13 +163,13 @@ __host__ __device__ constexpr int plane_c(int n1) { return n1 >= 256 ? 8 : n1 >=
 template <int N1, int N2>
 static cudaError_t plane_pass_impl(const PlaneArgs &a, cudaStream_t s) {
     static bool attr_done = false;
-    const bool overlap = a.planes * N1 * N2 < OVERLAP_POINTS;
+    const bool overlap = a.count * N1 * N2 < OVERLAP_POINTS;
     if constexpr (plane_solo(N1, N2)) {
         using P = Solo<N1, N2>;
-        return launch_cluster(k_solo_pass<N1, N2>, overlap, a.planes, 1, P::THREADS, P::SMEM, a, s, attr_done);
+        return launch_cluster(k_solo_pass<N1, N2>, overlap, a.count, 1, P::THREADS, P::SMEM, a, s, attr_done);
     } else {
         using P = Plane2<N1, N2, plane_c(N1), 1>;
-        return launch_cluster(k_plane_pass<N1, N2, plane_c(N1)>, overlap, a.planes, plane_c(N1), P::THREADS, P::SMEM, a, s,
+        return launch_cluster(k_plane_pass<N1, N2, plane_c(N1)>, overlap, a.count, plane_c(N1), P::THREADS, P::SMEM, a, s,
                               attr_done);
     }
 }
@@ -179,7 +179,7 @@ static cudaError_t solo_whole_impl(const PlaneArgs &a, cudaStream_t s) {
     if constexpr (plane_solo(N1, N2)) {
         using P = Solo<N1, N2>;
         static bool attr_done = false;
-        return launch_cluster(k_solo_whole<N1, N2>, true, a.instances, 1, P::THREADS, P::SMEM, a, s, attr_done);
+        return launch_cluster(k_solo_whole<N1, N2>, true, a.count, 1, P::THREADS, P::SMEM, a, s, attr_done);
     } else {
         return cudaErrorInvalidValue;
     }
@@ -188,7 +188,7 @@ static cudaError_t solo_whole_impl(const PlaneArgs &a, cudaStream_t s) {
 template <int N1, int N2, int C = plane_c(N1), int MINB = 2>
 static cudaError_t plane_whole_impl(const PlaneArgs &a, cudaStream_t s) {
     static bool attr_done = false;
-    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, true, a.instances, C, PLANE_THREADS, PlaneCfg<N1, N2, C>::SMEM, a, s,
+    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, true, a.count, C, PLANE_THREADS, PlaneCfg<N1, N2, C>::SMEM, a, s,
                           attr_done);
 }
 

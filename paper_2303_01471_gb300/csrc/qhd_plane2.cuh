@@ -362,19 +362,19 @@ __device__ __forceinline__ void solo_whole_run(const PlaneArgs &a, int64_t b, co
     constexpr int N2 = P::N2;
     float2 *g = a.psi + b * (int64_t)P::N1 * N2;
     const uint32_t *fq = a.fq + b * (int64_t)P::N1 * N2;
-    const float4 *tw_row = a.tw_row2 + P::V * TW2_TABLE * N2;
+    const float4 *tw_row = a.tw_row + P::V * TW2_TABLE * N2;
     plane2_copy<P, true>(tile, g, tid);
     __syncthreads();
 #pragma unroll 1
     for (int j = 0; j < a.cnt; ++j) {
-        solo_columns<P>(tile, j > 0, true, true, a.twc, fq, a.pot[(int64_t)j * a.batch + b],
+        solo_columns<P>(tile, j > 0, true, true, a.twx, fq, a.pot[(int64_t)j * a.batch + b],
                         step_dither(a.dither_base + (uint64_t)j), ptab, tid);
         __syncthreads();
         const float4 *kb = a.kt + ((int64_t)j * a.kt_batch + (a.kt_batch == 1 ? 0 : b)) * a.ksum;
         plane2_rows_kinetic<P>(tile, tw_row, kb, kb + P::N1, 0, tid);
         __syncthreads();
     }
-    solo_columns<P>(tile, a.cnt > 0, a.final_phase != 0, false, a.twc, fq, a.pot[(int64_t)a.cnt * a.batch + b], 0u, ptab,
+    solo_columns<P>(tile, a.cnt > 0, a.final_phase != 0, false, a.twx, fq, a.pot[(int64_t)a.cnt * a.batch + b], 0u, ptab,
                     tid);
     __syncthreads();
     plane2_copy<P, false>(tile, g, tid);
