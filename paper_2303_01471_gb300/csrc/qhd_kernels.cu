@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 4) k_row(RowArgs a) {
     using Sync = std::conditional_t<(T > 32), BlockSync, WarpSync>;
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
-    grid_release();
+    grid_release_upto(TINY_GRID);
     load_phase_tab(ptab, a.ptab);
     __syncthreads();
     const int line = threadIdx.x / T, t = threadIdx.x % T;
@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 4) k_row(RowArgs a) {
         x[e] = apply_phase_tab2(x[e], turns_mul(c, __ldg(&fq[i])) + a.dither, turns_mul(c, __ldg(&fq[N + i])) + a.dither,
                                 ptab);
     }
+    grid_release_upto(SMALL_GRID);
     if (a.mode & MODE_FWD) line_fft2<N, V, false>(x, sm, t, tw, Sync{}, at);
     if (valid) {
 #pragma unroll
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 4) k_row(RowArgs a) {
             g[N + t + T * e] = c2_second(x[e]);
         }
     }
+    grid_release();
 }
 
 // ------------------------------------------------------ strided axis pass
@@ -114,7 +116,9 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
     const int64_t ci = tile * (2 * CP) + 2 * c;
     float4 *g = reinterpret_cast<float4 *>(a.psi + o * (int64_t)N * a.inner + ci);
     const int64_t stride = a.inner / 2;
-    grid_release();
+    // tiny blocks in several waves leave even room everywhere
+    if (T == 1 && gridDim.x > 152 * 8) grid_release();
+    grid_release_upto(TINY_GRID);
     grid_wait();
     c2 x[E];
 #pragma unroll
@@ -176,6 +180,7 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
         // the mean's part: N mu = sum through the factor of frequency 0
         if (split0 && t == 0) st_c2(slot, c2_mul<false>(c2_mul_shared<false>(ld_c2(slot), kb[0]), kc));
     }
+    grid_release_upto(SMALL_GRID);
     if (a.mode & MODE_INV) line_fft2<N, V, true>(x, sm, t, tw, BlockSync{}, at);
     if (split0) {
         // written by the column's thread 0 before the inverse transform's barriers
@@ -188,6 +193,7 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
         const float2 p = c2_first(x[e]), q = c2_second(x[e]);
         g[(int64_t)(t + T * e) * stride] = make_float4(p.x, p.y, q.x, q.y);
     }
+    grid_release();
 }
 
 // --------------------------------------------- 1-D: a whole chunk per launch
@@ -261,7 +267,6 @@ __global__ void k_prep(PrepArgs a) {
     const int64_t b = blockIdx.y;
     __shared__ uint64_t s_k[3];
     __shared__ double s_fd[3];
-    grid_release();
     uint64_t pot = 0;
     if (threadIdx.x == 0) pot = prep_coefficients(a, jl, b, s_k, s_fd);
     __syncthreads();
@@ -272,10 +277,12 @@ __global__ void k_prep(PrepArgs a) {
     const float4 first = one ? prep_kinetic_entry(a, threadIdx.x, s_k, s_fd) : make_float4(0.f, 0.f, 0.f, 0.f);
     grid_wait();
     if (threadIdx.x == 0) a.pot[jl * a.batch + b] = pot;
-    if (!one) return;
-    float4 *out = a.kt + (jl * a.kt_batch + b) * a.ksum;
-    out[threadIdx.x] = first;
-    for (int i = threadIdx.x + blockDim.x; i < a.ksum; i += blockDim.x) out[i] = prep_kinetic_entry(a, i, s_k, s_fd);
+    if (one) {
+        float4 *out = a.kt + (jl * a.kt_batch + b) * a.ksum;
+        out[threadIdx.x] = first;
+        for (int i = threadIdx.x + blockDim.x; i < a.ksum; i += blockDim.x) out[i] = prep_kinetic_entry(a, i, s_k, s_fd);
+    }
+    grid_release();
 }
 
 // ------------------------------------------------------------ small kernels

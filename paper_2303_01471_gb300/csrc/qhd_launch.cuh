@@ -3,10 +3,25 @@
 // A small grid's pass is a few microseconds long, and between two passes of a
 // stream the GPU drains, launches and refills for one to two of them.  With
 // programmatic stream serialization the next grid's blocks are placed as soon
-// as every block of the previous grid has started (grid_release) and SM
-// resources come free; they do what depends on no earlier kernel (index
-// arithmetic, the static tables) and then wait for the previous grid's
-// completion (grid_wait).
+// as every block of the previous grid has released it (grid_release) or ended;
+// they do what depends on no earlier kernel (index arithmetic, the static tables)
+// and then wait for the previous grid's completion (grid_wait).
+//
+// Where a kernel releases decides where the next one's blocks land.  Released at the
+// start, they take the room that the running blocks leave, several to an SM while
+// others stay empty: kernels of about one block per SM then take up to twice as
+// long, and k_plane_whole, placed behind k_prep, keeps that for a whole chunk (per
+// step, released at the start / at the end / without overlap: 256^2 x 8 19.8 / 13.0 /
+// 13.1 us, 128x256 x 30 19.3 / 12.5 / 12.7, 64^3 17.1 / 9.8 / 14.7, 64x16x128 x 5
+// 17.5 / 15.1 / 22.8).  So the passes and k_prep release at their end, with these
+// exceptions.  A grid of up to 16 blocks is in nobody's way and releases at its start
+// (16x1024 x 1 6.4 us, 7.2 at the end); one of up to a block per SM before its last
+// transform (256x16 x 1 6.1 and 6.6, 128x16 x 4 5.4 and 6.1; with more threads than
+// that the early blocks get in the way again: 512x256 x 4 13.2 and 11.3); blocks of
+// one warp in many waves at their start (4x1024 x 300 15.6 and 17.7).  The
+// observables, k_uniform and the whole-run kernels, whose next kernel is k_prep or
+// the observables, release at their start (k_solo_whole, which clusters may follow,
+// at its end).
 //
 // Rules: every kernel launched through launch_overlapped calls grid_wait in all
 // its threads before it touches anything an earlier kernel writes, or writes
@@ -28,14 +43,26 @@
 namespace qhd {
 
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Released by grids of at most `threads` threads.
+__device__ __forceinline__ void grid_release_upto(unsigned threads) {
+    if (gridDim.x * blockDim.x <= threads) grid_release();
+}
+constexpr unsigned TINY_GRID = 16 * 128, SMALL_GRID = 152 * 128;
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Passes over fewer points than this overlap.  Measured per step, with and
-// without: 64x16x128 x 5 19.4 / 23.4 us, 512^2 x 16 48.8 / 53.6, 128^3 x 4 114.8 /
+// Passes over fewer points than this overlap.  Measured per step, with (released at
+// the start) and without: 64x16x128 x 5 19.4 / 23.4 us, 512^2 x 16 48.8 / 53.6, 128^3 x 4 114.8 /
 // 118.8, 512^2 x 32 95.9 / 101.1; at 2^24 points the gap no longer counts and
 // 256^3, whose plane and axis passes want different shared-memory splits of the
 // SM, loses: 257.8 / 244.5.
 constexpr int64_t OVERLAP_POINTS = int64_t(1) << 24;
+
+// Kernels that run a whole chunk overlap k_prep for chunks of up to this many steps:
+// the overlap saves 2.4 us per launch (64^2, chunks of 10 steps: 403 us per 100 steps,
+// 427 without), but a lone cluster placed while k_prep's last blocks run can be up to 9%
+// slower for all of its steps (128x256 x 1 7.11 us per step, 6.75 without; 256x32 x 1
+// 4.54 and 4.17).
+constexpr int OVERLAP_STEPS = 32;
 
 template <typename... P, typename... A>
 cudaError_t launch_overlapped(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

@@ -44,7 +44,6 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     const uint32_t *fq = a.fq + plane * (int64_t)N1 * N2;
     const float4 *tw_row = a.tw_row + P::V * TW2_TABLE * N2;
     const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
-    grid_release();
     load_phase_tab(ptab, a.ptab);
     grid_wait();
     const uint64_t coef = a.pot[plane >> a.log_planes];
@@ -55,6 +54,7 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     __syncthreads();
     if (fwd) plane2_rows_global<P, false>(tile, g, tw_row, tid);
     else plane2_copy<P, false>(tile, g, tid);
+    grid_release();
 }
 
 template <int N1, int N2, int C>
@@ -73,7 +73,6 @@ __global__ void __launch_bounds__(Plane2<N1, N2, C, 1>::THREADS, plane2_min_bloc
     const float4 *tw_row = a.tw_row + P::V * TW2_TABLE * N2;
     const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
     const uint32_t *fq = a.fq + plane * (int64_t)N1 * N2;
-    grid_release();
     load_phase_tab(ptab, a.ptab);
     grid_wait();
     const uint64_t coef = a.pot[plane >> a.log_planes];
@@ -94,6 +93,7 @@ __global__ void __launch_bounds__(Plane2<N1, N2, C, 1>::THREADS, plane2_min_bloc
     } else {
         plane2_copy<P, false>(tile, g, tid);
     }
+    grid_release();
 }
 
 template <int N1, int N2>
@@ -102,10 +102,10 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
     ulonglong2 *tile = reinterpret_cast<ulonglong2 *>(smem4 + PHASE_TAB);
-    grid_release();
     load_phase_tab(ptab, a.ptab);
     grid_wait();
     solo_whole_run<P>(a, blockIdx.x, ptab, tile, (int)threadIdx.x);
+    grid_release();
 }
 
 // MINB: CTAs per SM the kernel is compiled for (2 for batches; 1 for the wide
@@ -179,7 +179,8 @@ static cudaError_t solo_whole_impl(const PlaneArgs &a, cudaStream_t s) {
     if constexpr (plane_solo(N1, N2)) {
         using P = Solo<N1, N2>;
         static bool attr_done = false;
-        return launch_cluster(k_solo_whole<N1, N2>, true, a.count, 1, P::THREADS, P::SMEM, a, s, attr_done);
+        return launch_cluster(k_solo_whole<N1, N2>, a.cnt <= OVERLAP_STEPS, a.count, 1, P::THREADS, P::SMEM, a, s,
+                              attr_done);
     } else {
         return cudaErrorInvalidValue;
     }
@@ -188,8 +189,8 @@ static cudaError_t solo_whole_impl(const PlaneArgs &a, cudaStream_t s) {
 template <int N1, int N2, int C = plane_c(N1), int MINB = 2>
 static cudaError_t plane_whole_impl(const PlaneArgs &a, cudaStream_t s) {
     static bool attr_done = false;
-    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, true, a.count, C, PLANE_THREADS, PlaneCfg<N1, N2, C>::SMEM, a, s,
-                          attr_done);
+    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, a.cnt <= OVERLAP_STEPS, a.count, C, PLANE_THREADS,
+                          PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
 }
 
 bool plane_supported(int n1, int n2) {

@@ -78,3 +78,28 @@ def test_one_step_calls_match_one_call(shape, own_kinetic):
         sim.close()
     for a, b in zip(*states):
         assert np.max(np.abs(align_global_phase(b, a) - a)) <= ROUNDING * np.abs(a).max()
+
+
+# one launch of up to 16 blocks, of up to one block per SM, of more, and of one-warp
+# blocks in several waves: where a pass releases the next differs (csrc/qhd_launch.cuh);
+# chunks of 32 and of 33 steps: the whole-run kernels overlap or not
+@pytest.mark.parametrize("shape,batch", [((16, 16), 1), ((256, 16), 1), ((512, 64), 4), ((512, 64), 16), ((4, 1024), 300),
+                                         ((64, 64), 8), ((128, 128), 200), ((256, 256), 8), ((64, 64, 64), 1), ((64,), 64)],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+@pytest.mark.parametrize("steps", [32, 33])
+def test_repeated_runs_are_the_same_bits(shape, batch, steps):
+    """A pass that reads what the one before has not finished writing differs from run
+    to run: six runs queued without a synchronisation in between, each from a fresh
+    state, leave the same bits."""
+    sim = qhd.QHD(shape, batch=batch)
+    f = torch.rand((batch, *shape), dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    sim.set_potential(f)
+    sim.set_schedule(qhd.Schedule())
+    states = []
+    for _ in range(6):
+        sim.reset_state()
+        sim.evolve(steps * 0.01, 0.01)
+        states.append(sim.psi.clone())
+    assert all(torch.equal(s, states[0]) for s in states[1:])
+    assert abs(sim.observables()[-1].norm - 1.0) < 1e-5
+    sim.close()
