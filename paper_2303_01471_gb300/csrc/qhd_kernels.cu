@@ -94,6 +94,10 @@ __global__ void __launch_bounds__(ROW_THREADS, 4) k_row(RowArgs a) {
 // Lines of length N at stride `inner`; a block owns CP adjacent pairs of columns
 // of one plane, lanes run along the pairs, so each 16-byte access moves both
 // columns of a pair and each row of a tile is 16 CP contiguous bytes.
+// FLAT: a plane has fewer than CP pairs, and a block takes several planes' (the
+// last block what is left); with one plane per block such passes ran on blocks of
+// inner / 2 * T threads (1024x8x8 x 256, whose axis 1 had blocks of 4 threads: 816 us
+// per step, 366 with full ones).
 // Resident blocks: 4 of 128 threads with 8 points per thread; 3 with 16 (at 4,
 // the 128 registers a thread may then use spill: 256^3 axis-0 pass 69 us, 66 at 3).
 template <int N, int V, int CP> constexpr int axis_min_blocks() {
@@ -101,7 +105,7 @@ template <int N, int V, int CP> constexpr int axis_min_blocks() {
     return threads < 128 ? 1 : (Line2<N, V>::E == 16 ? 3 : 4) * 128 / threads;
 }
 
-template <int N, int V, int CP>
+template <int N, int V, int CP, bool FLAT>
 __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>()) k_axis(AxisArgs a) {
     using C = Line2<N, V>;
     using B = ColBuf<N, V, CP>;
@@ -111,9 +115,19 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
     const int c = threadIdx.x % CP, t = threadIdx.x / CP;
     constexpr int LOG_W = CP == 32 ? 6 : CP == 16 ? 5 : CP == 8 ? 4 : CP == 4 ? 3 : CP == 2 ? 2 : 1;  // log2(2 CP)
     static_assert(1 << LOG_W == 2 * CP, "tile width");
-    const int64_t o = blockIdx.x >> (a.log_inner - LOG_W);
-    const int64_t tile = blockIdx.x - (o << (a.log_inner - LOG_W));
-    const int64_t ci = tile * (2 * CP) + 2 * c;
+    int64_t o, tile, ci;
+    if (FLAT) {
+        const int64_t pair = (int64_t)blockIdx.x * CP + c;
+        o = pair >> (a.log_inner - 1);
+        tile = 0;
+        ci = 2 * (pair - (o << (a.log_inner - 1)));
+    } else {
+        o = blockIdx.x >> (a.log_inner - LOG_W);
+        tile = blockIdx.x - (o << (a.log_inner - LOG_W));
+        ci = tile * (2 * CP) + 2 * c;
+    }
+    const bool valid = !FLAT || o < a.planes;
+    if (!valid) o = 0;
     float4 *g = reinterpret_cast<float4 *>(a.psi + o * (int64_t)N * a.inner + ci);
     const int64_t stride = a.inner / 2;
     // tiny blocks in several waves leave even room everywhere
@@ -123,7 +137,7 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
     c2 x[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        const float4 v = g[(int64_t)(t + T * e) * stride];
+        const float4 v = valid ? g[(int64_t)(t + T * e) * stride] : make_float4(0.f, 0.f, 0.f, 0.f);
         x[e] = c2_make(make_float2(v.x, v.y), make_float2(v.z, v.w));
     }
     ulonglong2 *sm = reinterpret_cast<ulonglong2 *>(smem4) + c * B::S;
@@ -135,7 +149,7 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
     // same order.  The sum, later its part of the result, waits in a slot behind
     // the buffer, so that no other tile's pass holds registers for it.
     constexpr int ALL3 = MODE_FWD | MODE_KIN | MODE_INV;
-    const bool split0 = (a.mode & ALL3) == ALL3 && tile == 0;
+    const bool split0 = (a.mode & ALL3) == ALL3 && tile == 0;  // FLAT: every block has a column 0
     ulonglong2 *slot = reinterpret_cast<ulonglong2 *>(smem4) + (C::STAGES > 1 ? CP * B::S : 0) + c;
     if (split0) {
         ulonglong2 *red = reinterpret_cast<ulonglong2 *>(smem4);
@@ -188,10 +202,12 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
 #pragma unroll
         for (int e = 0; e < E; ++e) x[e] = x[e] + mean_part;
     }
+    if (valid) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const float2 p = c2_first(x[e]), q = c2_second(x[e]);
-        g[(int64_t)(t + T * e) * stride] = make_float4(p.x, p.y, q.x, q.y);
+        for (int e = 0; e < E; ++e) {
+            const float2 p = c2_first(x[e]), q = c2_second(x[e]);
+            g[(int64_t)(t + T * e) * stride] = make_float4(p.x, p.y, q.x, q.y);
+        }
     }
     grid_release();
 }
@@ -477,29 +493,24 @@ __host__ __device__ constexpr int axis_cp(int n, int t) {
     return n == 512 ? 4 : t >= 64 ? 2 : 128 / t > 32 ? 32 : 128 / t;
 }
 
-template <int N, int V, int CP>
-static cudaError_t axis_cp_impl(const AxisArgs &a, cudaStream_t s) {
+template <int N, int V, bool FLAT>
+static cudaError_t axis_tile_impl(const AxisArgs &a, cudaStream_t s) {
     using C = Line2<N, V>;
-    const int64_t blocks = a.planes * (a.inner / (2 * CP));
+    constexpr int CP = axis_cp(N, C::T);
+    const int64_t blocks = FLAT ? (a.planes * (a.inner / 2) + CP - 1) / CP : a.planes * (a.inner / (2 * CP));
     // exchange buffer (the zero-mode split's CP T partial sums use it too), then
     // that split's slot per pair
     constexpr size_t xch = ((C::STAGES > 1 ? (size_t)CP * ColBuf<N, V, CP>::S : 0) + CP) * sizeof(ulonglong2);
     static_assert(xch <= 48 * 1024, "default shared-memory limit");
     AxisArgs r = a;
     r.tw2 += V * TW2_TABLE * N;
-    return launch_overlapped(a.planes * a.inner * N < OVERLAP_POINTS, k_axis<N, V, CP>, dim3((unsigned)blocks),
+    return launch_overlapped(a.planes * a.inner * N < OVERLAP_POINTS, k_axis<N, V, CP, FLAT>, dim3((unsigned)blocks),
                              dim3(CP * C::T), xch, s, r);
 }
 
 template <int N, int V>
 static cudaError_t axis_v_impl(const AxisArgs &a, cudaStream_t s) {
-    constexpr int CP = axis_cp(N, Line2<N, V>::T);
-    if (a.inner >= 2 * CP) return axis_cp_impl<N, V, CP>(a, s);
-    if constexpr (CP > 16) if (a.inner >= 32) return axis_cp_impl<N, V, 16>(a, s);
-    if constexpr (CP > 8) if (a.inner >= 16) return axis_cp_impl<N, V, 8>(a, s);
-    if constexpr (CP > 4) if (a.inner >= 8) return axis_cp_impl<N, V, 4>(a, s);
-    if constexpr (CP > 2) if (a.inner >= 4) return axis_cp_impl<N, V, 2>(a, s);
-    return axis_cp_impl<N, V, 1>(a, s);
+    return a.inner >= 2 * axis_cp(N, Line2<N, V>::T) ? axis_tile_impl<N, V, false>(a, s) : axis_tile_impl<N, V, true>(a, s);
 }
 
 template <int N>
