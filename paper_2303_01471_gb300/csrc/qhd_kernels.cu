@@ -247,7 +247,11 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
 }
 
 // --------------------------------------------- 1-D: a whole chunk per launch
-template <int N>
+// OVERLAP: launched to overlap k_prep, so the kinetic tables are read with plain
+// loads, as in k_axis; those wait for the exchanges before them, where __ldg may be
+// issued ahead (100 steps of 256 points: 259 us with plain loads, 248 with __ldg), so
+// chunks that do not overlap keep it.
+template <int N, bool OVERLAP>
 __global__ void __launch_bounds__(ROW_THREADS) k_oned(OneDArgs a) {
     using C = LineCfg<N>;
     constexpr int E = C::E, T = C::T;
@@ -284,14 +288,13 @@ __global__ void __launch_bounds__(ROW_THREADS) k_oned(OneDArgs a) {
         const float2 sum = line_sum_lanes<E, T>(x);
         sub_line_mean<N, E>(x, sum);
         line_fft<N, false>(x, sm, t, a.tw2, WarpSync{});
-        // plain loads, as in k_axis
         const float4 *kb = a.kt + ((int64_t)j * a.kt_batch + (a.kt_batch == 1 ? 0 : b)) * N;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const float4 k0 = kb[t + T * e];
+            const float4 k0 = OVERLAP ? kb[t + T * e] : __ldg(&kb[t + T * e]);
             x[e] = cmul_comp(x[e], make_float2(k0.x, k0.y), make_float2(k0.z, k0.w));
         }
-        const float4 z0 = kb[0];
+        const float4 z0 = OVERLAP ? kb[0] : __ldg(&kb[0]);
         const float2 mean_part = cmul_comp(sum, make_float2(z0.x, z0.y), make_float2(z0.z, z0.w));
         line_fft<N, true>(x, sm, t, a.tw2, WarpSync{});
 #pragma unroll
@@ -561,7 +564,9 @@ static cudaError_t oned_impl(const OneDArgs &a, cudaStream_t s) {
     const int lpb = ROW_THREADS / C::T;
     const int64_t blocks = (a.batch + lpb - 1) / lpb;
     const size_t sm = PHASE_TAB * sizeof(float4) + (C::TWO_STAGE ? (size_t)lpb * S * sizeof(float2) : 0);
-    return launch_overlapped(true, k_oned<N>, dim3((unsigned)blocks), dim3(ROW_THREADS), sm, s, a);
+    const dim3 grid((unsigned)blocks), block(ROW_THREADS);
+    return a.cnt <= OVERLAP_STEPS ? launch_overlapped(true, k_oned<N, true>, grid, block, sm, s, a)
+                                  : launch_overlapped(false, k_oned<N, false>, grid, block, sm, s, a);
 }
 
 #define QHD_DISPATCH_N(n, fn, ...)                        \
