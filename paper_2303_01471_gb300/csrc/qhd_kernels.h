@@ -62,9 +62,9 @@ struct AxisArgs {
                                // s / r + perm1_c * (s % r), r = 2^perm1_log_r; perm1_c = 0: natural
 };
 
-// Plane engine (qhd_plane.cu): N1 distributed over a cluster, N2 per row.  Kept small:
-// with 152 bytes of arguments instead of 144 the compiler holds less of a step in
-// registers (one 128x64 instance: 139 of them instead of 167, 2.82 us per step instead of 2.76).
+// Plane engine (qhd_plane.cu): N1 distributed over a cluster, N2 per row.  Up to 144
+// bytes of arguments the compiler loads into registers once, longer ones it reads
+// where they are used (PlaneArgsLong, for the shapes where that is faster).
 struct PlaneArgs {
     float2 *psi;
     const uint32_t *fq;
@@ -86,6 +86,9 @@ struct PlaneArgs {
     int64_t kt_batch;        // whole: 1 = shared kinetic table, else batch
 };
 static_assert(sizeof(PlaneArgs) <= 144, "costs the cluster engine registers");
+struct PlaneArgsLong : PlaneArgs {
+    char unused[48];
+};
 
 struct OneDArgs {
     float2 *psi;

@@ -110,8 +110,18 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
 
 // MINB: CTAs per SM the kernel is compiled for (2 for batches; 1 for the wide
 // split, which runs only when every CTA has an SM of its own).
+// Args: PlaneArgsLong for the shapes that spill with the arguments in registers.  Per
+// step, in registers / in constant memory: 32x256 x 30 9.70 / 7.30 us, 64x128 x 60 9.81 /
+// 8.47, 256x64 x 60 13.1 / 12.8, 256x128 x 456 146.6 / 143.8; against 32x128 x 30 5.91 /
+// 6.07, 64^2 x 30 3.04 / 3.12, 128x64 x 1 2.86 / 2.91, 128x256 x 1 6.66 / 6.82, 256x32 x
+// 38 8.53 / 8.70, and no difference elsewhere.
+template <int N1, int N2, int C>
+using WholeArgs = std::conditional_t<(N1 == 32 && N2 == 256) || (N1 == 64 && N2 == 128 && C == 2) ||
+                                         (N1 == 256 && (N2 == 64 || N2 == 128)),
+                                     PlaneArgsLong, PlaneArgs>;
+
 template <int N1, int N2, int C, int MINB>
-__global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(PlaneArgs a) {
+__global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(WholeArgs<N1, N2, C> a) {
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
     float2 *tile = reinterpret_cast<float2 *>(smem4 + PHASE_TAB);
@@ -125,8 +135,8 @@ __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(PlaneArgs a
 }
 
 // ---------------------------------------------------------------- launchers
-template <typename K>
-static cudaError_t launch_cluster(K kernel, bool overlap, int64_t clusters, int c, int threads, size_t smem,
+template <typename Args>
+static cudaError_t launch_cluster(void (*kernel)(Args), bool overlap, int64_t clusters, int c, int threads, size_t smem,
                                   const PlaneArgs &a, cudaStream_t s, bool &attr_done) {
     if (!attr_done) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -152,7 +162,9 @@ static cudaError_t launch_cluster(K kernel, bool overlap, int64_t clusters, int 
     }
     cfg.attrs = attr;
     cfg.numAttrs = (unsigned)k;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
+    Args args{};
+    static_cast<PlaneArgs &>(args) = a;
+    return cudaLaunchKernelEx(&cfg, kernel, args);
 }
 
 // Cluster size per distributed-axis length: R = 32 rows per CTA (16 for 32).
