@@ -418,17 +418,8 @@ qhd_status qhd_init_grid(qhd_ctx **out, int ndim, const int64_t *n, const double
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
             if (wide && batch * (int64_t)wide <= (int64_t)sms) {
                 c->plane_c = wide;
-            } else if (plane_fits_solo((int)n[0], (int)n[1])) {
-                // One CTA per instance for whole waves of the GPU; what is left over
-                // runs on clusters if those fill at most two CTAs per SM (128^2: a solo
-                // wave of 152 takes 18.6 us per step, 152 instances on clusters 26.6, but
-                // 60 instances 10.3; 64^2: 456 14.8 / 19.9, and 152 12.6 / 6.7).
-                // A single wave with a few instances left over gains too little to pay
-                // for the second launch (128^2 x 160: 28.5 us, on clusters 26.8).
-                const int64_t wave = (int64_t)sms * solo_per_sm((int)n[0], (int)n[1]);
-                const int64_t left = batch % wave;
-                c->solo = left * c->plane_c <= 2 * (int64_t)sms ? batch - left : batch;
-                if (c->solo == wave && left > 0 && 7 * left < wave) c->solo = 0;
+            } else {
+                c->solo = solo_instances((int)n[0], (int)n[1], batch, sms);
                 if (c->solo > 0) c->plane_c = 1;
             }
         }

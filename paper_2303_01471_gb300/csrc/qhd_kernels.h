@@ -158,7 +158,7 @@ cudaError_t launch_plane_whole(int n1, int n2, const PlaneArgs &a, cudaStream_t 
 cudaError_t launch_solo_whole(int n1, int n2, const PlaneArgs &a, cudaStream_t s);
 bool plane_supported(int n1, int n2);
 bool plane_fits_solo(int n1, int n2);  // one CTA holds the plane
-int solo_per_sm(int n1, int n2);       // instances an SM runs at once in the solo form
+int64_t solo_instances(int n1, int n2, int64_t batch, int sms);  // 2-D: how many of a batch run in one CTA each
 int plane_cluster(int n1);
 // Whole-run kernel with twice the CTAs per instance (distributed axis 64 or 128; 0: none).
 int plane_cluster_wide(int n1);

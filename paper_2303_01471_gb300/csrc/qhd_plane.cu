@@ -238,7 +238,8 @@ template <int N1, int N2> static int solo_per_sm_of() {
     default: return cudaErrorInvalidValue;                                            \
     }
 
-int solo_per_sm(int n1, int n2) {
+// Instances an SM runs at once in the one-CTA form.
+static int solo_per_sm(int n1, int n2) {
     switch (n1 * 1000 + n2) {
     case 32032: return solo_per_sm_of<32, 32>();
     case 32064: return solo_per_sm_of<32, 64>();
@@ -251,9 +252,62 @@ int solo_per_sm(int n1, int n2) {
     case 128032: return solo_per_sm_of<128, 32>();
     case 128064: return solo_per_sm_of<128, 64>();
     case 128128: return solo_per_sm_of<128, 128>();
-    case 128256: return solo_per_sm_of<128, 256>();
     default: return 0;
     }
+}
+
+// Microseconds per step of a batch of n1 x n2 instances in the two forms (152 SMs,
+// 200 steps): tail, the first of few instances behind full waves of clusters; c1 and
+// c2, clusters on up to one and two CTAs per SM; solo[k - 1], one CTA each with k
+// instances per SM.
+struct FormTimes {
+    int n1, n2;
+    float tail, c1, c2, solo[6];
+};
+constexpr FormTimes FORM_TIMES[] = {
+    {32, 32, 2.16f, 2.96f, 3.60f, {5.84f, 7.16f, 8.65f, 10.47f, 12.95f, 15.18f}},
+    {32, 64, 3.12f, 3.44f, 4.41f, {6.23f, 8.45f, 11.02f}},
+    {32, 128, 5.67f, 6.25f, 7.45f, {6.20f}},
+    {32, 256, 5.70f, 7.70f, 10.67f, {10.54f}},
+    {64, 32, 3.18f, 3.87f, 4.78f, {5.14f, 6.87f, 9.51f, 12.28f, 15.19f, 18.07f}},
+    {64, 64, 3.76f, 5.48f, 6.76f, {6.12f, 10.32f, 14.79f}},
+    {64, 128, 6.13f, 8.52f, 10.97f, {10.41f}},
+    {64, 256, 9.75f, 12.72f, 18.75f, {18.87f}},
+    {128, 32, 2.90f, 3.36f, 4.28f, {8.36f, 10.78f, 15.94f, 25.40f}},
+    {128, 64, 4.28f, 5.08f, 6.48f, {9.84f, 17.38f}},
+    {128, 128, 5.93f, 7.70f, 10.95f, {18.48f}},
+};
+
+// How many of a batch's instances (the first ones) run in one CTA each: all, none,
+// or the whole waves of that form with the rest on clusters, whichever the times
+// above make shortest.  A split has to win by 8%: it costs a second launch, and its two
+// parts round differently.  Measured with every choice forced: 128^2 x 100 17.7 us on
+// clusters, 18.2 in one CTA each; x 120 21.4 / 18.3; x 512 74.5 / 72.6, split 65.4; 64^2 x
+// 78 6.05 / 5.60; 32^2 x 200 6.26 / 6.50, x 400 10.2 / 8.3; 128x32 x 78 7.67 / 7.32, x 152
+// 11.7 / 8.4; 64x256 x 304 36.8 / 37.3.  Batches of 8 instances per SM and more stay in
+// one CTA each where that is up to 4% behind (64x256 x 1216 143.8 / 148.9).
+int64_t solo_instances(int n1, int n2, int64_t batch, int sms) {
+    if (!plane_fits_solo(n1, n2)) return 0;
+    const FormTimes *f = FORM_TIMES;
+    while (f->n1 != n1 || f->n2 != n2) ++f;
+    const int c = plane_c(n1), per_sm = solo_per_sm(n1, n2);
+    // pairs of CTAs find room on every SM, clusters of four not quite (74 of 76)
+    const int64_t wave_c = 2 * (int64_t)sms / c - (c > 2 ? 2 : 0);
+    const double spread = c > 2 ? 0.8 : 1.0;  // share of the SMs up to which CTAs are alone on theirs
+    auto clusters = [&](int64_t b) {
+        const int64_t full = b / wave_c, rem = b % wave_c;
+        if (rem == 0) return (double)full * f->c2;
+        const double load = (double)(rem * c) / sms;
+        if (load > spread) return (double)(full + 1) * f->c2;
+        return full * f->c2 + (full ? f->tail + (f->c1 - f->tail) * load / spread : (double)f->c1);
+    };
+    const int64_t wave_s = (int64_t)sms * per_sm, full = batch / wave_s, rem = batch % wave_s;
+    const double whole = (double)full * f->solo[per_sm - 1];
+    const double solo = whole + (rem ? f->solo[(rem + sms - 1) / sms - 1] : 0.f);
+    const double split = full && rem ? whole + clusters(rem) : INFINITY;
+    const double limit = clusters(batch) * (batch >= 8 * (int64_t)sms ? 1.04 : 1.0);
+    if (split * 1.08 <= solo || solo > limit) return split <= limit ? full * wave_s : 0;
+    return batch;
 }
 
 cudaError_t launch_plane_pass(int n1, int n2, const PlaneArgs &a, cudaStream_t s) {

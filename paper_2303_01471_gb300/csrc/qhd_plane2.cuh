@@ -63,10 +63,11 @@ template <int N1_, int N2_, int C_, int V_> struct Plane2 {
 
 // Solo form: 16 points of a row pair per thread (plan 1) where that leaves no
 // thread idle in the row phase (64x128 x 512: 39.9 us per step with 8 points, 52.8
-// with 16 and half of the threads idle).
+// with 16 and half of the threads idle); rows of 256 points with 8 (64x256 x 1216 148.9,
+// 151.9 with 16).
 template <int N1, int N2> constexpr int solo_row_plan() {
     using P = Plane2<N1, N2, 1, 1>;
-    return P::RP * P::T2 >= P::THREADS ? 1 : 0;
+    return N2 < 256 && P::RP * P::T2 >= P::THREADS ? 1 : 0;
 }
 template <int N1, int N2> using Solo = Plane2<N1, N2, 1, solo_row_plan<N1, N2>()>;
 
