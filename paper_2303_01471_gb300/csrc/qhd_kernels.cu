@@ -164,8 +164,8 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
     if (!valid) o = 0;
     float4 *g = reinterpret_cast<float4 *>(a.psi + o * (int64_t)N * a.inner + ci);
     const int64_t stride = a.inner / 2;
-    // tiny blocks in several waves leave even room everywhere
-    if (T == 1 && gridDim.x > 152 * 8) grid_release();
+    // so many one-warp blocks leave even room everywhere
+    if (T == 1 && gridDim.x > 152 * 24) grid_release();
     grid_release_upto(TINY_GRID);
     grid_wait();
     c2 x[E];

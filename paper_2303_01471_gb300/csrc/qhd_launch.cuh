@@ -17,8 +17,9 @@
 // exceptions.  A grid of up to 16 blocks is in nobody's way and releases at its start
 // (16x1024 x 1 6.4 us, 7.2 at the end); one of up to a block per SM before its last
 // transform (256x16 x 1 6.1 and 6.6, 128x16 x 4 5.4 and 6.1; with more threads than
-// that the early blocks get in the way again: 512x256 x 4 13.2 and 11.3); blocks of
-// one warp in many waves at their start (4x1024 x 300 15.6 and 17.7).  The
+// that the early blocks get in the way again: 512x256 x 4 13.2 and 11.3); more than 24
+// one-warp blocks per SM at their start (4x1024 x 300 15.6 and 17.7; not with 13 per
+// SM, 8x128x256 x 4 25.9 and 17.3).  The
 // observables, k_uniform and the whole-run kernels, whose next kernel is k_prep or
 // the observables, release at their start (k_solo_whole, which clusters may follow,
 // at its end).
