@@ -475,9 +475,10 @@ static qhd_status set_potential_common(qhd_ctx *c) {
     const int64_t B = c->batch, G = c->g;
     const int nb = c->L.mm_blocks;
     QHD_LAUNCH(c, launch_minmax(c->f64, G, B, c->mm, nb, c->stream));
-    // few partials are cheaper to copy than one more kernel (64^2: 44 us against 50
-    // for the call), many are not (128^2 x 512, 1 MB of them: 449 against 402)
-    const bool on_device = nb * B > 1024;
+    // few partials are cheaper to copy than one more kernel (64^2 x 160, 2560 of them: 77
+    // us for the call, 88 with the kernel), many are not (128^2 x 512, 32768: 449 and 402);
+    // 5000 to 6000 are even
+    const bool on_device = nb > 1 && nb * B > 6144;
     const MinMaxPart *from = c->mm + (on_device ? nb * B : 0);
     if (on_device) QHD_LAUNCH(c, launch_minmax_final(c->mm, nb, B, c->mm + nb * B, c->stream));
     const int per = on_device ? 1 : nb;
