@@ -15,7 +15,6 @@
 #include "qhd_device.cuh"
 #include "qhd_group.h"
 #include "qhd_kernels.h"
-#include "qhd_packed.cuh"
 #include "qhd_trace.h"
 #include "qhd_sched.cuh"
 #include "qhd_spectrum.h"
@@ -348,57 +347,48 @@ qhd_status qhd_init_grid(qhd_ctx **out, int ndim, const int64_t *n, const double
     c->obs_res = (double *)(c->work + L.obs_res);
     c->mm = (MinMaxPart *)(c->work + L.mm);
 
-    // stage-2 twiddles per axis, tw2[m*R1 + j] = exp(-2 pi i j m / N) from FP64,
-    // stored as the FP32 value and its FP32 rounding residual
+    // twiddles from FP64, stored as the FP32 value and its FP32 rounding residual.
+    // Scalar line FFT, per axis: stage 2, tw[m * R1 + j] = exp(-2 pi i j m / N).  Packed
+    // line FFT, both plans, one table per stage after the first: entry [m * L + j] =
+    // exp(-2 pi i j m / (L R)), L the product of the radices before the stage, R its
+    // radix.  All are among the N-th roots of unity, which are computed once per length
+    // (a sine and a cosine per entry were most of the call: a 1024-point context 183 us,
+    // 158 so).
     std::vector<float4> tw((size_t)c->ksum, make_float4(0.f, 0.f, 0.f, 0.f));
-    for (int d = 0; d < ndim; ++d) {
-        int r1 = 0, r2 = 0;
-        plan_of((int)n[d], &r1, &r2);
-        c->tw[d] = (float4 *)(c->work + L.tw) + c->koff[d];
-        if (r2 <= 1) continue;
-        for (int m = 0; m < r2; ++m)
-            for (int j = 0; j < r1; ++j) {
-                const int64_t jm = ((int64_t)j * m) % n[d];
-                const double ang = 2.0 * 3.141592653589793238462643383279502884 * (double)jm / (double)n[d];
-                const double cr = cos(ang), ci = -sin(ang);
-                const float hr = (float)cr, hi = (float)ci;
-                tw[(size_t)c->koff[d] + (size_t)(m * r1 + j)] =
-                    make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
-            }
-    }
-    // twiddles of the packed line FFT, both plans, one table per stage after the
-    // first: entry [m * L + j] = exp(-2 pi i j m / (L R)), L the product of the
-    // radices before the stage, R its radix
     std::vector<float4> tw2((size_t)(2 * TW2_TABLE * c->ksum), make_float4(0.f, 0.f, 0.f, 0.f));
+    std::vector<float4> root;
     for (int d = 0; d < ndim; ++d) {
+        const int64_t N = n[d];
         const size_t first = (size_t)(2 * TW2_TABLE) * (size_t)c->koff[d];
+        c->tw[d] = (float4 *)(c->work + L.tw) + c->koff[d];
         c->tw2[d] = (float4 *)(c->work + L.tw2) + first;
         int same = 0;  // an earlier axis of this length has the same tables
-        while (n[same] != n[d]) ++same;
+        while (n[same] != N) ++same;
         if (same < d) {
-            const float4 *src = tw2.data() + (size_t)(2 * TW2_TABLE) * (size_t)c->koff[same];
-            std::copy(src, src + 2 * TW2_TABLE * n[d], tw2.begin() + (std::ptrdiff_t)first);
+            std::copy_n(&tw[(size_t)c->koff[same]], N, &tw[(size_t)c->koff[d]]);
+            std::copy_n(&tw2[(size_t)(2 * TW2_TABLE) * (size_t)c->koff[same]], 2 * TW2_TABLE * N, &tw2[first]);
             continue;
         }
+        root.resize((size_t)N);
+        for (int64_t k = 0; k < N; ++k) {
+            const double ang = 2.0 * 3.141592653589793238462643383279502884 * (double)k / (double)N;
+            const double cr = cos(ang), ci = -sin(ang);
+            const float hr = (float)cr, hi = (float)ci;
+            root[(size_t)k] = make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
+        }
+        int r1 = 0, r2 = 0;
+        plan_of((int)N, &r1, &r2);
+        if (r2 > 1)
+            for (int64_t i = 0; i < N; ++i) tw[(size_t)(c->koff[d] + i)] = root[(size_t)((i % r1) * (i / r1) % N)];
         for (int v = 0; v < 2; ++v) {
             int radix[4], stages = 0;
-            plan2_of((int)n[d], v, radix, &stages);
-            size_t at = first + (size_t)(v * TW2_TABLE) * (size_t)n[d];
-            if (v == 1 && !two_plans((int)n[d])) {  // one plan under both numbers
-                std::copy(tw2.begin() + (std::ptrdiff_t)first, tw2.begin() + (std::ptrdiff_t)at,
-                          tw2.begin() + (std::ptrdiff_t)at);
-                continue;
-            }
+            plan2_of((int)N, v, radix, &stages);
+            size_t at = first + (size_t)(v * TW2_TABLE) * (size_t)N;
             int64_t l = radix[0];
             for (int st = 1; st < stages; l *= radix[st], ++st) {
                 const int64_t period = l * radix[st];
-                for (int64_t i = 0; i < period; ++i) {
-                    const double ang = 2.0 * 3.141592653589793238462643383279502884 *
-                                       (double)(((i % l) * (i / l)) % period) / (double)period;
-                    const double cr = cos(ang), ci = -sin(ang);
-                    const float hr = (float)cr, hi = (float)ci;
-                    tw2[at++] = make_float4(hr, hi, (float)(cr - (double)hr), (float)(ci - (double)hi));
-                }
+                for (int64_t i = 0; i < period; ++i)
+                    tw2[at++] = root[(size_t)((i % l) * (i / l) % period * (N / period))];
             }
         }
     }
