@@ -315,11 +315,14 @@ __global__ void __launch_bounds__(ROW_THREADS) k_oned(OneDArgs a) {
 // Schedule evaluation at the step midpoints, the merged potential coefficients
 // and the per-axis kinetic phase tables of one chunk of steps (qhd_prep.cuh).
 
+// EARLY: releases the next kernel at the start (qhd_launch.cuh).
+template <bool EARLY>
 __global__ void k_prep(PrepArgs a) {
     const int64_t jl = blockIdx.x;  // local step 0..cnt (cnt is the extra potential entry)
     const int64_t b = blockIdx.y;
     __shared__ uint64_t s_k[3];
     __shared__ double s_fd[3];
+    if (EARLY) grid_release();
     uint64_t pot = 0;
     if (threadIdx.x == 0) pot = prep_coefficients(a, jl, b, s_k, s_fd);
     __syncthreads();
@@ -335,7 +338,7 @@ __global__ void k_prep(PrepArgs a) {
         out[threadIdx.x] = first;
         for (int i = threadIdx.x + blockDim.x; i < a.ksum; i += blockDim.x) out[i] = prep_kinetic_entry(a, i, s_k, s_fd);
     }
-    grid_release();
+    if (!EARLY) grid_release();
 }
 
 // ------------------------------------------------------------ small kernels
@@ -590,7 +593,8 @@ cudaError_t launch_oned(int n, const OneDArgs &a, cudaStream_t s) { QHD_DISPATCH
 
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
     dim3 grid((unsigned)(a.cnt + 1), (unsigned)a.batch);
-    return launch_overlapped(true, k_prep, grid, dim3(256), 0, s, a);
+    return launch_overlapped(true, a.batch == 1 && a.cnt > OVERLAP_STEPS ? k_prep<true> : k_prep<false>, grid, dim3(256), 0, s,
+                             a);
 }
 
 cudaError_t launch_uniform(float2 *psi, int64_t count, float value, cudaStream_t s) {

@@ -43,7 +43,8 @@
 
 namespace qhd {
 
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// No order with memory accesses is needed: the next kernel waits for this grid's end.
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }
 // Released by grids of at most `threads` threads.
 __device__ __forceinline__ void grid_release_upto(unsigned threads) {
     if (gridDim.x * blockDim.x <= threads) grid_release();
@@ -60,10 +61,12 @@ constexpr int64_t OVERLAP_POINTS = int64_t(1) << 24;
 
 // Kernels that run a whole chunk overlap k_prep for chunks of up to this many steps:
 // the overlap saves 2.4 us per launch (64^2, chunks of 10 steps: 403 us per 100 steps,
-// 427 without), but a lone cluster placed while k_prep's last blocks run can be up to 9%
-// slower for all of its steps (128x256 x 1 7.11 us per step, 6.75 without; 256x32 x 1
-// 4.54 and 4.17).  1-D, 64 points, 100 steps in chunks of 10: 228 us, 246 without; in
-// one chunk 140 and 131.
+// 427 without), but clusters placed while k_prep's last blocks run can be slower for
+// all of their steps (128x256 7.11 us per step, 6.75 without; 256x32 4.54 and 4.17).
+// 1-D, 64 points, 100 steps in chunks of 10: 228 us, 246 without; in one chunk 140 and
+// 131.  One instance alone is the exception: in plain order its cluster always lands on
+// the same SMs, good ones or bad ones by GPU (128^2 x 200 steps, 888 to 950 us on eight
+// GPUs); k_prep releases it at the start and it takes what is free (886 to 898).
 constexpr int OVERLAP_STEPS = 32;
 
 template <typename... P, typename... A>

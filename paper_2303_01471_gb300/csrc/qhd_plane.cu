@@ -112,12 +112,13 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
 // split, which runs only when every CTA has an SM of its own).
 // Args: PlaneArgsLong for the shapes that spill with the arguments in registers.  Per
 // step, in registers / in constant memory: 32x256 x 30 9.70 / 7.30 us, 64x128 x 60 9.81 /
-// 8.47, 256x64 x 60 13.1 / 12.8, 256x128 x 456 146.6 / 143.8; against 32x128 x 30 5.91 /
+// 8.47, 256x64 x 60 13.1 / 12.8, 256x128 x 456 146.6 / 143.8, 256^2 x 60 40.2 / 39.7, 128^2 on
+// 8 CTAs 4.64 / 4.59; against 32x128 x 30 5.91 /
 // 6.07, 64^2 x 30 3.04 / 3.12, 128x64 x 1 2.86 / 2.91, 128x256 x 1 6.66 / 6.82, 256x32 x
 // 38 8.53 / 8.70, and no difference elsewhere.
 template <int N1, int N2, int C>
 using WholeArgs = std::conditional_t<(N1 == 32 && N2 == 256) || (N1 == 64 && N2 == 128 && C == 2) ||
-                                         (N1 == 256 && (N2 == 64 || N2 == 128)),
+                                         (N1 == 128 && N2 == 128 && C == 8) || (N1 == 256 && N2 >= 64),
                                      PlaneArgsLong, PlaneArgs>;
 
 template <int N1, int N2, int C, int MINB>
@@ -201,7 +202,7 @@ static cudaError_t solo_whole_impl(const PlaneArgs &a, cudaStream_t s) {
 template <int N1, int N2, int C = plane_c(N1), int MINB = 2>
 static cudaError_t plane_whole_impl(const PlaneArgs &a, cudaStream_t s) {
     static bool attr_done = false;
-    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, a.cnt <= OVERLAP_STEPS, a.count, C, PLANE_THREADS,
+    return launch_cluster(k_plane_whole<N1, N2, C, MINB>, a.cnt <= OVERLAP_STEPS || a.batch == 1, a.count, C, PLANE_THREADS,
                           PlaneCfg<N1, N2, C>::SMEM, a, s, attr_done);
 }
 
