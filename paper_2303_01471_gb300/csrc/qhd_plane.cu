@@ -96,6 +96,17 @@ __global__ void __launch_bounds__(Plane2<N1, N2, C, 1>::THREADS, plane2_min_bloc
     grid_release();
 }
 
+// A block's instance.  HIDDEN: the compiler cannot tell that the index is a small
+// unsigned number and keeps fewer of a step's addresses in registers, which spill in
+// some shapes.
+template <bool HIDDEN> __device__ __forceinline__ int64_t instance_of(unsigned i) {
+    int64_t zero = 0;
+    if (HIDDEN) asm volatile("" : "+l"(zero));
+    return zero + i;
+}
+
+// Hidden index: per step, without / with, 32x256 x 608 41.3 / 39.7 us, 64x32 x 304 6.86 /
+// 6.74; against 128^2 x 608 72.3 / 74.9, 64^2 x 304 10.3 / 10.4.
 template <int N1, int N2>
 __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1, N2>>()) k_solo_whole(PlaneArgs a) {
     using P = Solo<N1, N2>;
@@ -104,22 +115,25 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     ulonglong2 *tile = reinterpret_cast<ulonglong2 *>(smem4 + PHASE_TAB);
     load_phase_tab(ptab, a.ptab);
     grid_wait();
-    solo_whole_run<P>(a, blockIdx.x, ptab, tile, (int)threadIdx.x);
+    solo_whole_run<P>(a, instance_of<N2 == 256 || N2 == 32>(blockIdx.x), ptab, tile, (int)threadIdx.x);
     grid_release();
 }
 
 // MINB: CTAs per SM the kernel is compiled for (2 for batches; 1 for the wide
 // split, which runs only when every CTA has an SM of its own).
-// Args: PlaneArgsLong for the shapes that spill with the arguments in registers.  Per
-// step, in registers / in constant memory: 32x256 x 30 9.70 / 7.30 us, 64x128 x 60 9.81 /
-// 8.47, 256x64 x 60 13.1 / 12.8, 256x128 x 456 146.6 / 143.8, 256^2 x 60 40.2 / 39.7, 128^2 on
-// 8 CTAs 4.64 / 4.59; against 32x128 x 30 5.91 /
-// 6.07, 64^2 x 30 3.04 / 3.12, 128x64 x 1 2.86 / 2.91, 128x256 x 1 6.66 / 6.82, 256x32 x
-// 38 8.53 / 8.70, and no difference elsewhere.
+// Args: PlaneArgsLong for shapes that spill with the arguments in registers.  Per
+// step, in registers / in constant memory: 64x128 x 60 9.81 / 8.47 us, 256x64 x 60 13.1 /
+// 12.8, 256x128 x 456 146.6 / 143.8, 128^2 on 8 CTAs 4.64 / 4.59; against 32x128 x 30 5.91 /
+// 6.07, 64^2 x 30 3.04 / 3.12, 128x64 x 1 2.86 / 2.91, 128x256 x 1 6.66 / 6.82, 256x32 x 38
+// 8.53 / 8.70.  Hidden index, without / with: 32x256 x 30 9.70 / 7.08, 256x128 x 456 143.8 /
+// 139.9 and x 1 8.57 / 8.02, 256^2 x 8 13.1 / 12.9; against 256x32 x 38 8.57 / 8.78, 128^2 x 30
+// 8.13 / 8.34.
 template <int N1, int N2, int C>
-using WholeArgs = std::conditional_t<(N1 == 32 && N2 == 256) || (N1 == 64 && N2 == 128 && C == 2) ||
-                                         (N1 == 128 && N2 == 128 && C == 8) || (N1 == 256 && N2 >= 64),
-                                     PlaneArgsLong, PlaneArgs>;
+using WholeArgs =
+    std::conditional_t<(N1 == 64 && N2 == 128 && C == 2) || (N1 == 128 && N2 == 128 && C == 8) ||
+                           (N1 == 256 && (N2 == 64 || N2 == 128)),
+                       PlaneArgsLong, PlaneArgs>;
+template <int N1, int N2> constexpr bool WHOLE_HIDDEN = (N1 == 32 && N2 == 256) || (N1 == 256 && N2 >= 128);
 
 template <int N1, int N2, int C, int MINB>
 __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(WholeArgs<N1, N2, C> a) {
@@ -132,7 +146,8 @@ __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_plane_whole(WholeArgs<N
 #pragma unroll
     for (int q = 0; q < C; ++q) tiles[q] = cluster_addr(tile, (uint32_t)q);
     grid_release();
-    plane_whole_run<N1, N2, C, 1>(a, blockIdx.x / C, rank, tiles, ptab, tile, true, cluster);
+    plane_whole_run<N1, N2, C, 1>(a, instance_of<WHOLE_HIDDEN<N1, N2>>(blockIdx.x / C), rank, tiles, ptab, tile, true,
+                                  cluster);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -269,8 +284,8 @@ constexpr FormTimes FORM_TIMES[] = {
     {32, 32, 2.16f, 2.96f, 3.60f, {5.84f, 7.16f, 8.65f, 10.47f, 12.95f, 15.18f}},
     {32, 64, 3.12f, 3.44f, 4.41f, {6.23f, 8.45f, 11.02f}},
     {32, 128, 5.67f, 6.25f, 7.45f, {6.20f}},
-    {32, 256, 5.70f, 7.70f, 10.67f, {10.54f}},
-    {64, 32, 3.18f, 3.87f, 4.78f, {5.14f, 6.87f, 9.51f, 12.28f, 15.19f, 18.07f}},
+    {32, 256, 5.70f, 7.50f, 10.67f, {10.06f}},
+    {64, 32, 3.18f, 3.87f, 4.78f, {5.14f, 6.74f, 9.43f, 12.14f, 15.19f, 18.07f}},
     {64, 64, 3.76f, 5.48f, 6.76f, {6.12f, 10.32f, 14.79f}},
     {64, 128, 6.13f, 8.52f, 10.97f, {10.41f}},
     {64, 256, 9.75f, 12.72f, 18.75f, {18.87f}},
