@@ -8,8 +8,10 @@
 //     the same arithmetic as the stand-alone prep kernel, qhd_prep.cuh);
 //   * instance items run every Strang step of the chunk for CL / sub instances
 //     of one context, each held in the shared memory of `sub` CTAs of the
-//     cluster (the whole-run engine of qhd_plane.cuh; sub = 1, for 64^2: the solo
-//     form of qhd_plane2.cuh).
+//     cluster (the whole-run engine of qhd_plane.cuh).
+// A context whose own form is one CTA per instance stays out of the queue: its own
+// launches run beside it, on a branch of the same graph, so that a group with the
+// default split gives every context the bits of its own qhd_evolve.
 // All prep items precede all instance items in the queue, and a cluster claims
 // an item only when it has finished the previous one, so when an instance item
 // waits for its context's tables, every prep item it needs has been claimed by
@@ -31,7 +33,6 @@
 #include "qhd_trace.h"
 #include "qhd_kernels.h"
 #include "qhd_plane.cuh"
-#include "qhd_plane2.cuh"
 #include "qhd_prep.cuh"
 
 namespace qhd {
@@ -113,17 +114,6 @@ __device__ __forceinline__ void group_run(const PlaneArgs &pa, int64_t b, bool l
     plane_whole_run<N, N, C, 1>(pa, b, r, tiles, ptab, tile, live, cluster);
 }
 
-// One CTA per instance (solo form): nothing is shared between the CTAs, so an
-// idle one has nothing to do.
-template <int N>
-__device__ __noinline__ void group_solo(const PlaneArgs &pa, int64_t b, bool live, float2 *tile, float4 *ptab) {
-    using P = Solo<N, N>;
-    static_assert(P::THREADS == PLANE_THREADS, "one instance per CTA");
-    load_phase_tab(ptab, pa.ptab);
-    __syncthreads();
-    if (live) solo_whole_run<P>(pa, b, ptab, reinterpret_cast<ulonglong2 *>(tile), (int)threadIdx.x);
-}
-
 // Instance item k of context c: wait for its tables, then every step of the
 // chunk for instances k * (CL / sub) + grp, grp = 0 .. CL / sub - 1.
 __device__ __forceinline__ void group_instance(const GroupArgs &a, const GroupClass &g, int c, int64_t k, int crank,
@@ -152,7 +142,6 @@ __device__ __forceinline__ void group_instance(const GroupArgs &a, const GroupCl
     const bool live = b < s_pa.batch;
     const int64_t bb = live ? b : s_pa.batch - 1;  // idle CTAs read a valid instance's tables
     switch (g.n * 16 + sub) {
-    case 64 * 16 + 1: group_solo<64>(s_pa, bb, live, tile, ptab); break;
     case 64 * 16 + 2: group_run<64, 2>(s_pa, bb, live, grp, r, tile, ptab, cluster); break;
     case 64 * 16 + 4: group_run<64, 4>(s_pa, bb, live, grp, r, tile, ptab, cluster); break;
     case 64 * 16 + 8: group_run<64, 8>(s_pa, bb, live, grp, r, tile, ptab, cluster); break;
@@ -204,7 +193,6 @@ __global__ void __launch_bounds__(PLANE_THREADS, MINB) k_group(GroupArgs a) {
 // Shared memory of one CTA for a (edge, CTAs per instance) class; 0: no such class.
 static size_t class_smem(int n, int sub) {
     switch (n * 16 + sub) {
-    case 64 * 16 + 1: return Solo<64, 64>::SMEM;
     case 64 * 16 + 2: return PlaneCfg<64, 64, 2>::SMEM;
     case 64 * 16 + 4: return PlaneCfg<64, 64, 4>::SMEM;
     case 64 * 16 + 8: return PlaneCfg<64, 64, 8>::SMEM;
@@ -240,14 +228,16 @@ using namespace qhd;
 
 struct qhd_group {
     std::vector<qhd_ctx *> ctxs;
-    std::vector<int> sub;            // CTAs per instance per context
+    std::vector<int> sub;            // CTAs per instance per context (in the queue)
+    std::vector<char> own_form;      // context runs its own launches beside the queue
     std::vector<int> edge;           // mesh edge per context
     int min_blocks = 2;
     int clusters = 0;
     size_t smem = 0;
     cudaStream_t stream = nullptr;   // the contexts' (caller's) stream
     cudaStream_t own = nullptr;      // private stream the graph is captured and replayed on
-    cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+    cudaStream_t side = nullptr;     // the branch of the contexts' own launches, in capture
+    cudaEvent_t ev_in = nullptr, ev_out = nullptr, ev_fork = nullptr, ev_join = nullptr;
     char *work = nullptr;
     GroupClass *d_cls = nullptr;     // [GROUP_MAX_CHUNKS][n_ctx]
     unsigned *d_count = nullptr;     // [GROUP_MAX_CHUNKS][1 + n_ctx] queue and arrivals
@@ -258,12 +248,16 @@ struct qhd_group {
     cudaGraphExec_t exec = nullptr;
     std::string key;
     int64_t launches = 0, captures = 0;
+    int64_t graph_launches = 0;      // kernels of the captured graph
     qhd_status sticky = QHD_OK;
     std::string err;
     ~qhd_group() {
         if (exec) cudaGraphExecDestroy(exec);
         if (ev_in) cudaEventDestroy(ev_in);
         if (ev_out) cudaEventDestroy(ev_out);
+        if (ev_fork) cudaEventDestroy(ev_fork);
+        if (ev_join) cudaEventDestroy(ev_join);
+        if (side) cudaStreamDestroy(side);
         if (own) cudaStreamDestroy(own);
     }
 };
@@ -362,17 +356,17 @@ qhd_status qhd_group_create(qhd_group **out, qhd_ctx *const *ctxs, int n_ctx, co
             return QHD_ERR_INVALID_ARG;
         }
         const int idx = v.n[0] == 64 ? 0 : v.n[0] == 128 ? 1 : 2;
-        // default: the context's own split, so the group runs its arithmetic; 128^2 in
-        // one CTA each wants 512 threads and an SM of its own, which the launch's
-        // clusters of two CTAs per SM do not give
+        // default: the context's own form, so the group runs its arithmetic
+        const bool own_form = !c.sub_cluster[idx] && v.plane_c == 1;
         int sub = c.sub_cluster[idx] ? c.sub_cluster[idx] : v.plane_c;
-        if (!c.sub_cluster[idx] && (sub == 0 || (sub == 1 && v.n[0] != 64))) sub = default_sub(v.n[0]);
-        if (c.sub_cluster[idx] == 1 || !sub_ok(v.n[0], sub)) {
+        if (own_form || sub == 0) sub = default_sub(v.n[0]);
+        if (!sub_ok(v.n[0], sub)) {
             delete g;
             return QHD_ERR_INVALID_ARG;
         }
         g->ctxs.push_back(ctxs[i]);
         g->sub.push_back(sub);
+        g->own_form.push_back(own_form);
         g->edge.push_back((int)v.n[0]);
         g->smem = std::max(g->smem, class_smem((int)v.n[0], sub));
     }
@@ -394,6 +388,11 @@ qhd_status qhd_group_create(qhd_group **out, qhd_ctx *const *ctxs, int n_ctx, co
     cudaError_t e = cudaStreamCreateWithFlags(&g->own, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->ev_in, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->ev_out, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming);
+    for (int i = 0; i < n_ctx && e == cudaSuccess; ++i)
+        if (g->own_form[(size_t)i]) e = ctx_whole_load(ctxs[i]);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem);
     if (e == cudaSuccess) {
         if (c.clusters > 0) {
@@ -452,6 +451,8 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
                  v.split, v.kinetic);
         key += kb;
     }
+    // an injected time-out is one of the queue's waits: every context runs there
+    auto beside = [&](int i) { return g->own_form[(size_t)i] && g->extra_wait == 0; };
     if (key != g->key || !g->exec) {
         g->key.clear();
         g->h_cls.assign((size_t)(n_chunks * n_ctx), GroupClass{});
@@ -460,6 +461,7 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
             const int64_t j0 = q * chunk, cnt = std::min(chunk, nsteps - j0);
             int64_t item = 0;
             for (int i = 0; i < n_ctx; ++i) {  // prep items first
+                if (beside(i)) continue;
                 GroupClass &gc = g->h_cls[(size_t)(q * n_ctx + i)];
                 gc.prep_first = item;
                 gc.prep_count = (cnt + 1 + GROUP_PREP_STEPS - 1) / GROUP_PREP_STEPS;
@@ -467,6 +469,7 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
                 item += gc.prep_count;
             }
             for (int i = 0; i < n_ctx; ++i) {
+                if (beside(i)) continue;
                 const GroupCtxView &v = views[(size_t)i];
                 GroupClass &gc = g->h_cls[(size_t)(q * n_ctx + i)];
                 const int sub = g->sub[(size_t)i], per = GROUP_CL / sub;
@@ -502,8 +505,8 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
                 pl.fq = v.fq;
                 pl.pot = v.pot;
                 pl.kt = v.kt;
-                pl.tw_row = sub > 1 ? v.tw_row : v.tw_row2;
-                pl.twx = sub > 1 ? g->d_twx + (size_t)i * GROUP_TWX : v.twc;
+                pl.tw_row = v.tw_row;
+                pl.twx = g->d_twx + (size_t)i * GROUP_TWX;
                 pl.batch = v.batch;
                 pl.cnt = (int)cnt;
                 pl.final_phase = j0 + cnt == nsteps ? 1 : 0;
@@ -520,12 +523,22 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
         QHD_GCUDA(g, cudaMemcpyAsync(g->d_cls, g->h_cls.data(), g->h_cls.size() * sizeof(GroupClass),
                                      cudaMemcpyHostToDevice, g->own));
         QHD_GCUDA(g, cudaStreamSynchronize(g->own));
-        // capture: per chunk, zero the queue and arrival counters, then the launch
+        // capture: per chunk, zero the queue and arrival counters, then the launch;
+        // beside them the launches of the contexts that stay out of the queue
+        g->graph_launches = 0;
         cudaGraph_t graph = nullptr;
         QHD_GCUDA(g, cudaStreamBeginCapture(g->own, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
         void *kern = group_kernel(g->min_blocks);
+        bool forked = false;
+        for (int i = 0; i < n_ctx; ++i) forked = forked || beside(i);
+        if (forked) {
+            e = cudaEventRecord(g->ev_fork, g->own);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(g->side, g->ev_fork, 0);
+            forked = e == cudaSuccess;
+        }
         for (int64_t q = 0; q < n_chunks && e == cudaSuccess; ++q) {
+            if (n_items[(size_t)q] == 0) continue;
             unsigned *cnt = g->d_count + q * (1 + n_ctx);
             e = cudaMemsetAsync(cnt, 0, sizeof(unsigned) * (size_t)(1 + n_ctx), g->own);
             if (e != cudaSuccess) break;
@@ -541,6 +554,17 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
             cudaLaunchConfig_t lc = group_launch_config(g->clusters, g->smem, g->own, attr);
             void *args[] = {&ga};
             e = cudaLaunchKernelExC(&lc, kern, args);
+            g->graph_launches++;
+        }
+        // the queue first: its clusters need several SMs of a GPC each, the branch's CTAs fill
+        // what is left (per step, 160 x 64^2 + 20 x 256^2: 33 us, 35 the other way round, 44 one
+        // after the other; 128 x 128^2 + 128 x 256^2 93, 108, 101)
+        for (int i = 0; i < n_ctx && e == cudaSuccess; ++i)
+            if (beside(i)) e = ctx_whole_enqueue(g->ctxs[(size_t)i], nsteps, dt, g->side, &g->graph_launches);
+        if (forked) {  // the branch joins whatever happened, or the capture could not end
+            const cudaError_t j = cudaEventRecord(g->ev_join, g->side);
+            const cudaError_t k = j == cudaSuccess ? cudaStreamWaitEvent(g->own, g->ev_join, 0) : j;
+            if (e == cudaSuccess) e = k;
         }
         cudaError_t e2 = cudaStreamEndCapture(g->own, &graph);
         if (e == cudaSuccess) e = e2;
@@ -565,7 +589,7 @@ qhd_status qhd_group_evolve(qhd_group *g, double T, double dt) {
     QHD_GCUDA(g, cudaGraphLaunch(g->exec, g->own));
     QHD_GCUDA(g, cudaEventRecord(g->ev_out, g->own));
     QHD_GCUDA(g, cudaStreamWaitEvent(g->stream, g->ev_out, 0));
-    g->launches += n_chunks;
+    g->launches += g->graph_launches;
     for (auto *c : g->ctxs) ctx_advance(c, nsteps, dt);
     return QHD_OK;
 }
@@ -600,7 +624,7 @@ qhd_status qhd_group_info(const qhd_group *g, int64_t *out) {
     for (size_t i = 0; i < 3; ++i) out[5 + i] = 0;
     for (size_t i = 0; i < g->ctxs.size(); ++i) {
         const int idx = g->edge[i] == 64 ? 0 : g->edge[i] == 128 ? 1 : 2;
-        out[5 + idx] = g->sub[i];
+        out[5 + idx] = g->own_form[i] ? 1 : g->sub[i];
     }
     return QHD_OK;
 }

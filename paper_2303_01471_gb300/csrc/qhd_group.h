@@ -19,7 +19,6 @@ struct GroupCtxView {
     const uint32_t *fq;
     uint64_t *pot;           // [chunk + 1][batch]
     float4 *kt;              // [chunk][kt_batch][ksum]
-    const float4 *tw_row2, *twc;  // packed row twiddles, column twiddles of the solo form
     const float4 *tw_row;    // stage-2 twiddles of axis 1
     const float4 *ptab;
     const SchedDev *sched;
@@ -36,6 +35,11 @@ struct GroupCtxView {
 
 // Fills v; QHD_ERR_STATE without a potential and a schedule.
 qhd_status ctx_group_view(qhd_ctx *c, GroupCtxView *v);
+// A context whose own form runs one CTA per instance (plane_c == 1): its launches of
+// an evolution by nsteps of dt on stream s, neither advancing its clock nor counting;
+// *launches grows by their number.  ctx_whole_load loads their kernels first.
+cudaError_t ctx_whole_load(const qhd_ctx *c);
+cudaError_t ctx_whole_enqueue(const qhd_ctx *c, int64_t nsteps, double dt, cudaStream_t s, int64_t *launches);
 // Advances the context's clock after a batched launch evolved it by nsteps of dt.
 void ctx_advance(qhd_ctx *c, int64_t nsteps, double dt);
 

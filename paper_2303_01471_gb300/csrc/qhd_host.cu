@@ -609,6 +609,61 @@ qhd_status qhd_get_time(const qhd_ctx *c, double *t_out, int64_t *steps_out) {
 
 namespace {
 
+// Step tables of an evolution by nsteps of dt; the caller fills in the chunk.
+PrepArgs prep_args(const qhd_ctx *c, int64_t nsteps, double dt) {
+    PrepArgs pa{};
+    pa.sched = c->sched;
+    pa.inst = c->inst;
+    pa.pot = c->pot;
+    pa.kt = c->kt;
+    pa.t_start = c->t;
+    pa.dt = dt;
+    pa.nsteps = nsteps;
+    pa.batch = c->batch;
+    pa.ndim = c->ndim;
+    for (int d = 0; d < 3; ++d) {
+        pa.n[d] = d < c->ndim ? (int)c->n[d] : 1;
+        pa.len[d] = d < c->ndim ? c->hi[d] - c->lo[d] : 1.0;
+        pa.koff[d] = d < c->ndim ? c->koff[d] : c->ksum;
+    }
+    pa.ksum = c->ksum;
+    pa.inv_g = 1.0 / (double)c->g;
+    pa.split = c->split == QHD_SPLIT_LIE_TROTTER ? 1 : 0;
+    pa.kinetic = c->kinetic == QHD_KINETIC_FD2 ? 1 : 0;
+
+    pa.kt_batch = c->kt_shared ? 1 : c->batch;
+    return pa;
+}
+
+// Arguments of a chunk's launches of the 2-D whole-run engine: of its one-CTA part
+// (the first c->solo instances) and of the rest, on clusters (the same arrays from its
+// first instance on).
+PlaneArgs whole_args(const qhd_ctx *c, const PrepArgs &pa, bool last_chunk, bool solo) {
+    PlaneArgs w{};
+    const int64_t first = solo ? 0 : c->solo;
+    w.psi = c->psi + first * c->g;
+    w.fq = c->fq + first * c->g;
+    w.pot = c->pot + first;
+    w.kt = c->kt + (pa.kt_batch > 1 ? first * c->ksum : 0);
+    w.tw_row = solo ? c->tw2[1] : c->tw[1];
+    w.twx = solo ? c->twc : c->twx;
+    w.count = solo ? c->solo : c->batch - c->solo;
+    w.batch = c->batch;
+    w.cnt = (int)pa.cnt;
+    w.final_phase = last_chunk ? 1 : 0;
+    w.ksum = c->ksum;
+    w.dither_base = (uint64_t)(c->steps_done + pa.j0);
+    w.ptab = c->ptab;
+    w.kt_batch = pa.kt_batch;
+    return w;
+}
+
+cudaError_t launch_whole(const qhd_ctx *c, const PlaneArgs &w, bool solo, cudaStream_t s) {
+    const int n0 = (int)c->n[0], n1 = (int)c->n[1];
+    if (solo) return launch_solo_whole(n0, n1, w, s);
+    return c->plane_c == plane_cluster_wide(n0) ? launch_plane_whole_wide(n0, n1, w, s) : launch_plane_whole(n0, n1, w, s);
+}
+
 // One chunk of steps with the tensor-core transform: per step a potential
 // split, W along axis 1, a transposing split, W along axis 0, the kinetic
 // split, conj W along axis 0, a transposing split, conj W along axis 1.  The
@@ -683,29 +738,9 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
     const int ndim = c->ndim;
     const int64_t B = c->batch;
 
-    PrepArgs pa{};
-    pa.sched = c->sched;
-    pa.inst = c->inst;
-    pa.pot = c->pot;
-    pa.kt = c->kt;
-    pa.t_start = c->t;
-    pa.dt = dt;
-    pa.nsteps = nsteps;
-    pa.batch = B;
-    pa.ndim = ndim;
-    for (int d = 0; d < 3; ++d) {
-        pa.n[d] = d < ndim ? (int)c->n[d] : 1;
-        pa.len[d] = d < ndim ? c->hi[d] - c->lo[d] : 1.0;
-        pa.koff[d] = d < ndim ? c->koff[d] : c->ksum;
-    }
-    pa.ksum = c->ksum;
-    pa.inv_g = 1.0 / (double)c->g;
-    pa.split = c->split == QHD_SPLIT_LIE_TROTTER ? 1 : 0;
-    pa.kinetic = c->kinetic == QHD_KINETIC_FD2 ? 1 : 0;
-
+    PrepArgs pa = prep_args(c, nsteps, dt);
     const int64_t ch = c->kt_shared ? c->L.chunk_shared : c->L.chunk;
-    const int64_t ktb = c->kt_shared ? 1 : B;
-    pa.kt_batch = ktb;
+    const int64_t ktb = pa.kt_batch;
     for (int64_t j0 = 0; j0 < nsteps; j0 += ch) {
         const int64_t cnt = nsteps - j0 < ch ? nsteps - j0 : ch;
         const bool last_chunk = j0 + cnt == nsteps;
@@ -739,38 +774,10 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
             continue;
         }
         if (c->plane_mode == 2) {
-            PlaneArgs w{};
-            w.psi = c->psi;
-            w.fq = c->fq;
-            w.pot = c->pot;
-            w.kt = c->kt;
-            w.batch = B;
-            w.cnt = (int)cnt;
-            w.final_phase = last_chunk ? 1 : 0;
-            w.ksum = c->ksum;
-            w.dither_base = (uint64_t)(c->steps_done + j0);
-            w.ptab = c->ptab;
-            w.kt_batch = ktb;
             TimedScope ts(c, QHD_KCLASS_WHOLE, true);
-            if (c->solo > 0) {
-                w.tw_row = c->tw2[1];
-                w.twx = c->twc;
-                w.count = c->solo;
-                QHD_LAUNCH(c, launch_solo_whole((int)c->n[0], (int)c->n[1], w, c->stream));
-                // the rest of the batch: the same arrays from its first instance on
-                w.psi += c->solo * c->g;
-                w.fq += c->solo * c->g;
-                w.pot += c->solo;
-                if (ktb > 1) w.kt += c->solo * c->ksum;
-            }
-            w.tw_row = c->tw[1];
-            w.twx = c->twx;
-            w.count = B - c->solo;
-            if (w.count > 0) {
-                if (c->plane_c == plane_cluster_wide((int)c->n[0]))
-                    QHD_LAUNCH(c, launch_plane_whole_wide((int)c->n[0], (int)c->n[1], w, c->stream));
-                else
-                    QHD_LAUNCH(c, launch_plane_whole((int)c->n[0], (int)c->n[1], w, c->stream));
+            for (const bool solo : {true, false}) {
+                const PlaneArgs w = whole_args(c, pa, last_chunk, solo);
+                if (w.count > 0) QHD_LAUNCH(c, launch_whole(c, w, solo, c->stream));
             }
             continue;
         }
@@ -1127,8 +1134,6 @@ qhd_status ctx_group_view(qhd_ctx *c, GroupCtxView *v) {
     v->pot = c->pot;
     v->kt = c->kt;
     v->tw_row = c->ndim >= 2 ? c->tw[1] : nullptr;
-    v->tw_row2 = c->ndim >= 2 ? c->tw2[1] : nullptr;
-    v->twc = c->twc;
     v->ptab = c->ptab;
     v->sched = c->sched;
     v->inst = c->inst;
@@ -1142,6 +1147,31 @@ qhd_status ctx_group_view(qhd_ctx *c, GroupCtxView *v) {
     v->whole_run = c->plane_mode == 2 && c->tc == nullptr;
     v->plane_c = c->plane_mode == 2 ? c->plane_c : 0;
     return QHD_OK;
+}
+
+cudaError_t ctx_whole_load(const qhd_ctx *c) {
+    const PlaneArgs none{};  // no instances: the kernels are loaded, nothing is launched
+    cudaError_t e = load_prep();
+    if (e == cudaSuccess) e = launch_whole(c, none, true, nullptr);
+    return e == cudaSuccess ? launch_whole(c, none, false, nullptr) : e;
+}
+
+cudaError_t ctx_whole_enqueue(const qhd_ctx *c, int64_t nsteps, double dt, cudaStream_t s, int64_t *launches) {
+    PrepArgs pa = prep_args(c, nsteps, dt);
+    const int64_t ch = c->kt_shared ? c->L.chunk_shared : c->L.chunk;
+    for (pa.j0 = 0; pa.j0 < nsteps; pa.j0 += ch) {
+        pa.cnt = std::min(ch, nsteps - pa.j0);
+        cudaError_t e = launch_prep(pa, s);
+        ++*launches;
+        for (const bool solo : {true, false}) {
+            const PlaneArgs w = whole_args(c, pa, pa.j0 + pa.cnt == nsteps, solo);
+            if (e != cudaSuccess || w.count == 0) continue;
+            e = launch_whole(c, w, solo, s);
+            ++*launches;
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 void ctx_advance(qhd_ctx *c, int64_t nsteps, double dt) {

@@ -602,6 +602,12 @@ cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
                              a);
 }
 
+cudaError_t load_prep() {
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, k_prep<true>);
+    return e == cudaSuccess ? cudaFuncGetAttributes(&fa, k_prep<false>) : e;
+}
+
 cudaError_t launch_uniform(float2 *psi, int64_t count, float value, cudaStream_t s) {
     int64_t blocks = (count + 255) / 256;
     if (blocks > 152 * 32) blocks = 152 * 32;

@@ -146,6 +146,8 @@ cudaError_t launch_row(int n, const RowArgs &a, cudaStream_t s);
 cudaError_t launch_axis(int n, const AxisArgs &a, cudaStream_t s);
 cudaError_t launch_oned(int n, const OneDArgs &a, cudaStream_t s);
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s);
+// Loads launch_prep's kernels (a first launch inside a stream capture must not).
+cudaError_t load_prep();
 cudaError_t launch_uniform(float2 *psi, int64_t count, float value, cudaStream_t s);
 cudaError_t launch_minmax(const double *f, int64_t g, int64_t batch, MinMaxPart *part, int nblk,
                           cudaStream_t s);

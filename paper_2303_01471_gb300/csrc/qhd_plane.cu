@@ -159,6 +159,7 @@ static cudaError_t launch_cluster(void (*kernel)(Args), bool overlap, int64_t cl
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
+    if (clusters == 0) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * c), 1, 1);
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
