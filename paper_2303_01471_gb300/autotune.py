@@ -26,7 +26,7 @@ from . import qhd
 CACHE_DIR = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tune")
 CACHE_FILE = os.path.join(CACHE_DIR, "group.json")
 
-# CTAs per instance allowed for each mesh edge (the engine holds at most 32 rows per CTA)
+# CTAs per instance in the queue for each mesh edge (the engine holds at most 32 rows per CTA)
 SUB_CHOICES = {64: (2, 4, 8), 128: (4, 8), 256: (8,)}
 EDGE_SLOT = {64: 0, 128: 1, 256: 2}
 
@@ -47,7 +47,10 @@ def cache_key(sims) -> str:
 
 def candidates(sims) -> List[qhd.GroupConfig]:
     edges = sorted({s.shape[0] for s in sims})
-    per_edge = [SUB_CHOICES[e] for e in edges]
+    # contexts whose own form is one CTA per instance: that form, which only the default
+    # (0) gives, is a candidate too
+    solo = {s.shape[0] for s in sims if getattr(s, "cluster_ctas", int)() == 1}
+    per_edge = [((0,) if e in solo else ()) + SUB_CHOICES[e] for e in edges]
     out = []
     for subs in itertools.product(*per_edge):
         sub = [0, 0, 0]
