@@ -774,10 +774,11 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
             continue;
         }
         if (c->plane_mode == 2) {
-            TimedScope ts(c, QHD_KCLASS_WHOLE, true);
             for (const bool solo : {true, false}) {
                 const PlaneArgs w = whole_args(c, pa, last_chunk, solo);
-                if (w.count > 0) QHD_LAUNCH(c, launch_whole(c, w, solo, c->stream));
+                if (w.count == 0) continue;
+                TimedScope ts(c, QHD_KCLASS_WHOLE, true);
+                QHD_LAUNCH(c, launch_whole(c, w, solo, c->stream));
             }
             continue;
         }
