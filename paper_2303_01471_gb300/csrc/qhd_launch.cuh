@@ -69,6 +69,13 @@ constexpr int64_t OVERLAP_POINTS = int64_t(1) << 24;
 // GPUs); k_prep releases it at the start and it takes what is free (886 to 898).
 constexpr int OVERLAP_STEPS = 32;
 
+// A launch's error is its caller's to report: it does not stay behind as the thread's
+// last error, where the next plain launch, of any context, would find it.
+inline cudaError_t launched(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 template <typename... P, typename... A>
 cudaError_t launch_overlapped(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               A... args) {
@@ -82,7 +89,7 @@ cudaError_t launch_overlapped(bool overlap, void (*kernel)(P...), dim3 grid, dim
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    return launched(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
 }
 
 }  // namespace qhd

@@ -181,7 +181,7 @@ static cudaError_t launch_cluster(void (*kernel)(Args), bool overlap, int64_t cl
     cfg.numAttrs = (unsigned)k;
     Args args{};
     static_cast<PlaneArgs &>(args) = a;
-    return cudaLaunchKernelEx(&cfg, kernel, args);
+    return launched(cudaLaunchKernelEx(&cfg, kernel, args));
 }
 
 // Cluster size per distributed-axis length: R = 32 rows per CTA (16 for 32).
