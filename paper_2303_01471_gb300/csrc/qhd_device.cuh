@@ -183,10 +183,10 @@ template <int N> struct LineCfg {
 __host__ __device__ constexpr int pad_index(int i, int log_r1) { return i + (i >> log_r1); }
 
 // Worst shared-memory bank conflict (8-byte words, evaluated per half warp)
-// of the two exchange patterns for a line stride S.  lanes: lane l works on
-// line (ROWMAJOR ? l / T : l % W) at thread index (ROWMAJOR ? l % T : l / W).
+// of the two exchange patterns for a line stride S; lane l works on line l / T at
+// thread index l % T.
 template <int N>
-__host__ __device__ constexpr int conflicts(int S, bool rowmajor, int W) {
+__host__ __device__ constexpr int conflicts(int S) {
     using C = LineCfg<N>;
     int worst = 1;
     for (int pass = 0; pass < 2; ++pass) {
@@ -197,8 +197,8 @@ __host__ __device__ constexpr int conflicts(int S, bool rowmajor, int W) {
                     int addr[16] = {};
                     for (int l = 0; l < 16; ++l) {
                         int lane = 16 * h + l;
-                        int line = rowmajor ? (C::T >= 32 ? 0 : lane / C::T) : lane % W;
-                        int t = rowmajor ? (C::T >= 32 ? lane : lane % C::T) : lane / W;
+                        int line = C::T >= 32 ? 0 : lane / C::T;
+                        int t = C::T >= 32 ? lane : lane % C::T;
                         if (t >= C::T) t %= C::T;
                         int j = t + C::T * q;
                         int i = pass == 0 ? j * C::R1 + m : j + m * C::R1;
@@ -216,14 +216,14 @@ __host__ __device__ constexpr int conflicts(int S, bool rowmajor, int W) {
     return worst;
 }
 
-// Best line stride (in float2) in [PADDED, PADDED + 16] for the lane layout.
+// Best line stride (in float2) in [PADDED, PADDED + 16].
 template <int N>
-__host__ __device__ constexpr int line_stride(bool rowmajor, int W) {
+__host__ __device__ constexpr int line_stride() {
     using C = LineCfg<N>;
     if (!C::TWO_STAGE) return 0;
     int best = C::PADDED, best_c = 1 << 30;
     for (int S = C::PADDED; S <= C::PADDED + 16; ++S) {
-        int c = conflicts<N>(S, rowmajor, W);
+        int c = conflicts<N>(S);
         if (c < best_c) {
             best_c = c;
             best = S;

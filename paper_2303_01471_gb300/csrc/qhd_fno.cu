@@ -380,36 +380,6 @@ __global__ void __launch_bounds__(FT) k_fno_frags(uint4 *dfty, uint4 *lay, uint4
     }
 }
 
-// Axis-1 truncated DFT stage of row bx from its bf16 pairs Vt[c][y pair] in shared
-// memory: each warp owns one 16 x 8 tile of D (k_fno_dfty_tc), the scaled result
-// goes out through Ds.  Called by the whole block.
-__device__ __forceinline__ void dfty_tile(const uint32_t *Vt, float *Ds, const Dims &d, int64_t bx, float s0, float s1,
-                                          float2 *out, const uint4 *fr) {
-    const int n = d.n, M = d.M, LDV = n / 2 + 4;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int r = lane / 4, q = 2 * (lane % 4);
-    const int mt = warp / 4, nt = warp % 4;  // 2 x 4 tiles of 16 x 8
-    float acc[4] = {};
-    const int ka = 16 * mt + r, kb = ka + 8, c = 8 * nt + r;
-    const uint4 *frm = fr + (size_t)mt * (n / 16) * 32 + lane;
-    for (int y0 = 0; y0 < n; y0 += 16) {
-        const int y = y0 + q;
-        const uint4 A = __ldg(&frm[(y0 / 16) * 32]);
-        mma_bf16(acc, A.x, A.y, A.z, A.w, Vt[c * LDV + y / 2], Vt[c * LDV + y / 2 + 4]);
-    }
-    const int co = 8 * nt + q;
-    Ds[ka * 33 + co] = acc[0];
-    Ds[ka * 33 + co + 1] = acc[1];
-    Ds[kb * 33 + co] = acc[2];
-    Ds[kb * 33 + co + 1] = acc[3];
-    __syncthreads();
-    for (int o = threadIdx.x; o < M * TC_C; o += blockDim.x) {
-        const int ky = o / TC_C, cc = o % TC_C;
-        const float sc = ky == 0 ? s0 : s1;
-        out[bx * (int64_t)M * TC_C + o] = make_float2(Ds[ky * 33 + cc] * sc, Ds[(16 + ky) * 33 + cc] * sc);
-    }
-}
-
 // Layer output of row bx = (b, x) on the tensor cores:
 //   a[y][o] = sum_c v[y][c] Ww[o][c] + sum_k T[y][k] U[k][o] + bw[o],
 //   T[y][k] = cos(2 pi k y / n) (k < 16), -sin(2 pi (k - 16) y / n) (k >= 16),
@@ -565,7 +535,7 @@ __global__ void __launch_bounds__(FT) k_fno_dfty_tc(const T *in, Dims d, float s
                                                     const uint4 *fr) {
     __shared__ uint32_t Vt[TC_C * (128 + 4)];  // [c][y pair], n <= 256
     __shared__ float Ds[32 * 33];
-    const int n = d.n, LDV = n / 2 + 4;
+    const int n = d.n, M = d.M, LDV = n / 2 + 4;
     const int64_t bx = blockIdx.x;
     const T *src = in + bx * (int64_t)n * TC_C;
     if constexpr (sizeof(T) == 2) {
@@ -594,7 +564,29 @@ __global__ void __launch_bounds__(FT) k_fno_dfty_tc(const T *in, Dims d, float s
         }
     }
     __syncthreads();
-    dfty_tile(Vt, Ds, d, bx, s0, s1, out, fr);
+    // each warp owns one 16 x 8 tile of D; the scaled result goes out through Ds
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int r = lane / 4, q = 2 * (lane % 4);
+    const int mt = warp / 4, nt = warp % 4;  // 2 x 4 tiles of 16 x 8
+    float acc[4] = {};
+    const int ka = 16 * mt + r, kb = ka + 8, c = 8 * nt + r;
+    const uint4 *frm = fr + (size_t)mt * (n / 16) * 32 + lane;
+    for (int y0 = 0; y0 < n; y0 += 16) {
+        const int y = y0 + q;
+        const uint4 A = __ldg(&frm[(y0 / 16) * 32]);
+        mma_bf16(acc, A.x, A.y, A.z, A.w, Vt[c * LDV + y / 2], Vt[c * LDV + y / 2 + 4]);
+    }
+    const int co = 8 * nt + q;
+    Ds[ka * 33 + co] = acc[0];
+    Ds[ka * 33 + co + 1] = acc[1];
+    Ds[kb * 33 + co] = acc[2];
+    Ds[kb * 33 + co + 1] = acc[3];
+    __syncthreads();
+    for (int o = threadIdx.x; o < M * TC_C; o += blockDim.x) {
+        const int ky = o / TC_C, cc = o % TC_C;
+        const float sc = ky == 0 ? s0 : s1;
+        out[bx * (int64_t)M * TC_C + o] = make_float2(Ds[ky * 33 + cc] * sc, Ds[(16 + ky) * 33 + cc] * sc);
+    }
 }
 
 // Backward of the layer input on the tensor cores (BF16 path), as k_fno_layer_in_bwd:

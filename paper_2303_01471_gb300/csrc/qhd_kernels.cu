@@ -255,7 +255,7 @@ template <int N, bool OVERLAP>
 __global__ void __launch_bounds__(ROW_THREADS) k_oned(OneDArgs a) {
     using C = LineCfg<N>;
     constexpr int E = C::E, T = C::T;
-    constexpr int S = line_stride<N>(true, 0);
+    constexpr int S = line_stride<N>();
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
     float2 *smem = reinterpret_cast<float2 *>(smem4 + PHASE_TAB);
@@ -435,9 +435,10 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
 }
 
 // FP64 bounds it (5.3e11 FMA/s on the whole GPU, 1/74 of the FP32 rate), so each
-// point costs only its own products: the squared coordinate distances to x* are one table per block, and the distance is
-// compared squared, with the largest square whose root is below the radius.  With
-// a square root and the coordinates' arithmetic per point, 256^3 took 897 us.
+// point costs only its own products: the squared coordinate distances to x* are one
+// table per block, and the distance is compared squared, with the largest square
+// whose root is below the radius.  256^3 with |psi|^2, the call: 932 us with a square
+// root and the coordinates' arithmetic per point, 449 so.
 __global__ void __launch_bounds__(256) k_obs_partial(ObsArgs a) {
     extern __shared__ double d2[];  // (x - x*)^2 per axis, at a.coff[d]
     const int64_t b = blockIdx.y;
@@ -568,7 +569,7 @@ static cudaError_t axis_impl(const AxisArgs &a, cudaStream_t s) {
 template <int N>
 static cudaError_t oned_impl(const OneDArgs &a, cudaStream_t s) {
     using C = LineCfg<N>;
-    constexpr int S = line_stride<N>(true, 0);
+    constexpr int S = line_stride<N>();
     const int lpb = ROW_THREADS / C::T;
     const int64_t blocks = (a.batch + lpb - 1) / lpb;
     const size_t sm = PHASE_TAB * sizeof(float4) + (C::TWO_STAGE ? (size_t)lpb * S * sizeof(float2) : 0);

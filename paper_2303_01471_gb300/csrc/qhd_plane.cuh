@@ -17,8 +17,8 @@
 // phase (diagonal in position space) and the forward step are fused with no
 // barrier between them: two cluster barriers per Strang step.
 //
-// This is the engine of 2-D instances that do not fit one CTA (256-point axes)
-// and of small batches, where the length of the chain of one step counts and not
+// This is the engine of 2-D instances that do not fit one CTA (256 points along axis
+// 0, or more than 16384 in all) and of small batches, where the length of the chain of one step counts and not
 // the throughput: scalar lines have the shorter one (one 128^2 instance on 8
 // CTAs 4.5 us per step, 6.0 us with packed pairs as in qhd_plane2.cuh).
 #pragma once
@@ -37,7 +37,7 @@ constexpr int PLANE_THREADS = 256;
 template <int N1, int N2, int C> struct PlaneCfg {
     static constexpr int R = N1 / C;                      // rows per CTA
     using RowC = LineCfg<N2>;
-    static constexpr int S = line_stride<N2>(true, 0);     // row stride in float2 (>= padded row)
+    static constexpr int S = line_stride<N2>();     // row stride in float2 (>= padded row)
     static constexpr int T2 = RowC::T, E2 = RowC::E;
     static constexpr int ROWS_PER_ITER = PLANE_THREADS / T2;
     static constexpr int PAIRS = (R / C) * N2;            // exchange positions owned per CTA

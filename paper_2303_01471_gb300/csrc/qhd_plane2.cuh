@@ -230,11 +230,12 @@ template <typename P> __device__ __noinline__ void plane2_zero_row_back(ulonglon
 // the line engine (its content is in registers at that point).
 template <typename P>
 __device__ __forceinline__ void plane2_rows_kinetic(ulonglong2 *tile, const float4 *__restrict__ tw_row,
-                                                    const float4 *kt0, const float4 *kt1, int rank, int tid) {
-    constexpr int T2 = P::T2, E2 = P::E2, N2 = P::N2, C = P::C, V = P::V;
+                                                    const float4 *kt0, const float4 *kt1, int tid) {
+    static_assert(P::C == 1, "solo form");
+    constexpr int T2 = P::T2, E2 = P::E2, N2 = P::N2, V = P::V;
     const RowAddr<Line2<N2, V>::LOG_R1> at;
     const int t = tid % T2;
-    if (rank == 0 && tid < T2) plane2_zero_row_out<P>(tile, kt0, kt1, t);
+    if (tid < T2) plane2_zero_row_out<P>(tile, kt0, kt1, t);
 #pragma unroll 1
     for (int base = 0; base < P::RP; base += P::PAIRS_PER_ITER) {
         const int p = base + tid / T2;
@@ -245,10 +246,9 @@ __device__ __forceinline__ void plane2_rows_kinetic(ulonglong2 *tile, const floa
             for (int e = 0; e < E2; ++e) x[e] = ld_c2(&rp[t + T2 * e]);
             __syncwarp();
             line_fft2<N2, V, false>(x, rp, t, tw_row, Warp2Sync{}, at);
-            // rows p and p + RP hold frequencies rank + C p and rank + C (p + RP)
-            // along the column axis; plain (coherent) loads: the batched persistent
-            // kernel writes these tables earlier in the same launch
-            const w2 k0 = w2_make(kt0[rank + C * p], kt0[rank + C * (p + P::RP)]);
+            // rows p and p + RP hold these frequencies along the column axis; plain
+            // loads: the step tables may still be written when the block starts
+            const w2 k0 = w2_make(kt0[p], kt0[p + P::RP]);
 #pragma unroll
             for (int e = 0; e < E2; ++e) x[e] = c2_mul_shared<false>(c2_mul<false>(x[e], k0), kt1[t + T2 * e]);
             line_fft2<N2, V, true>(x, rp, t, tw_row, Warp2Sync{}, at);
@@ -256,7 +256,7 @@ __device__ __forceinline__ void plane2_rows_kinetic(ulonglong2 *tile, const floa
             for (int e = 0; e < E2; ++e) st_c2(&rp[t + T2 * e], x[e]);
         }
     }
-    if (rank == 0 && tid < T2) plane2_zero_row_back<P>(tile, t);
+    if (tid < T2) plane2_zero_row_back<P>(tile, t);
 }
 
 // Rows along N2, one direction, between global memory and the tile: inverse reads
@@ -372,7 +372,7 @@ __device__ __forceinline__ void solo_whole_run(const PlaneArgs &a, int64_t b, co
                         step_dither(a.dither_base + (uint64_t)j), ptab, tid);
         __syncthreads();
         const float4 *kb = a.kt + ((int64_t)j * a.kt_batch + (a.kt_batch == 1 ? 0 : b)) * a.ksum;
-        plane2_rows_kinetic<P>(tile, tw_row, kb, kb + P::N1, 0, tid);
+        plane2_rows_kinetic<P>(tile, tw_row, kb, kb + P::N1, tid);
         __syncthreads();
     }
     solo_columns<P>(tile, a.cnt > 0, a.final_phase != 0, false, a.twx, fq, a.pot[(int64_t)a.cnt * a.batch + b], 0u, ptab,
