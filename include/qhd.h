@@ -257,11 +257,17 @@ int64_t qhd_library_call_count(const qhd_ctx *ctx);
  * plane (3-D plane passes) of the plane engine; 0 for the generic passes or a
  * NULL context.  For 2-D grids whose axis 0 has 64 or 128 points, a batch with at
  * most (SM count / wide split) instances runs on twice the default CTAs per
- * instance (4 for 64, 8 for 128: half the rows per CTA).  Batches that fill the
- * GPU several times over run their instances of up to 16384 points in one CTA
- * each (reported as 1; what does not fill a wave may still run on clusters).
- * Fixed at qhd_init_grid.  A batched group (qhd_group_*) uses the same split by
- * default (128^2: never less than 4). */
+ * instance (4 for 64, 8 for 128: half the rows per CTA).  Larger batches run
+ * instances of up to 128 rows and 16384 points in one CTA each where that is the
+ * faster form (reported as 1), some of them only their whole waves, the first
+ * instances, with the rest on clusters.  Fixed at qhd_init_grid.  A batched group
+ * (qhd_group_*) runs every context in its own form by default.
+ *
+ * Rounding: the forms, and the plans of the generic passes (chosen by the points of
+ * a launch), order their operations differently.  The same instance can therefore
+ * differ in its last bits between batches of different sizes, and between the first
+ * instances of a 2-D batch and those on clusters.  Repeating a call on the same
+ * batch repeats its bits. */
 int qhd_cluster_ctas(const qhd_ctx *ctx);
 
 /*
@@ -550,7 +556,10 @@ qhd_status qhd_lattice_destroy(qhd_lattice *lat);
  * steps: a grid of clusters of 8 CTAs pulls work items from a device queue,
  * first the step tables of each context, then groups of instances, each
  * instance held in the shared memory of `sub` CTAs of a cluster (8 / sub
- * instances per cluster item).  The launch sequence is captured once into a
+ * instances per cluster item).  Contexts whose own form is one CTA per instance
+ * (qhd_cluster_ctas = 1) stay out of the queue by default: their own launches run
+ * beside it on a branch of the same graph.  With the default split every context
+ * gets the bits of its own qhd_evolve.  The launch sequence is captured once into a
  * CUDA graph and replayed while T, dt and the contexts' clocks at the call
  * repeat (e.g. reset_state, group_evolve, observables, ...); a change
  * re-captures.  Waits for the tables are bounded: qhd_group_status
@@ -558,7 +567,8 @@ qhd_status qhd_lattice_destroy(qhd_lattice *lat);
  * also makes the group and its contexts sticky-failed.
  *
  * cfg (may be NULL for the defaults, every field 0): sub_cluster[k] = CTAs per
- * instance for edge 64 (k = 0: 2, 4 or 8), 128 (k = 1: 4 or 8), 256 (k = 2: 8);
+ * instance in the queue for edge 64 (k = 0: 2, 4 or 8), 128 (k = 1: 4 or 8), 256
+ * (k = 2: 8), 0 = each context's own form (one CTA per instance is only had so);
  * min_blocks = resident CTAs per SM the kernel is compiled for (1 or 2);
  * clusters = persistent clusters launched (0: as many as fit at once).  These
  * are the choices the benchmark's autotuner searches.
@@ -588,7 +598,8 @@ qhd_status qhd_group_status(qhd_group *g);
 qhd_status qhd_group_inject_wait_timeout(qhd_group *g, int on);
 /* out (8 values): clusters launched, min_blocks, shared memory per CTA (bytes),
  * kernel launches so far, graph captures so far, CTAs per instance for edge 64,
- * 128, 256 (0 when no context has that edge). */
+ * 128, 256 (0 when no context has that edge; 1: the context's own form, beside the
+ * queue). */
 qhd_status qhd_group_info(const qhd_group *g, int64_t *out);
 const char *qhd_group_last_error(const qhd_group *g); /* "" if none; g may be NULL */
 qhd_status qhd_group_destroy(qhd_group *g);

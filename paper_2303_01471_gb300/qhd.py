@@ -71,8 +71,9 @@ class _Schedule(ctypes.Structure):
 
 class GroupConfig(ctypes.Structure):
     """Launch choices of a batched group (qhd_group_config): CTAs per instance for
-    mesh edge 64 / 128 / 256 (0 = default 2 / 4 / 8), resident CTAs per SM the
-    kernel is compiled for (1 or 2, 0 = 2), persistent clusters (0 = all that fit)."""
+    mesh edge 64 (2, 4, 8) / 128 (4, 8) / 256 (8), 0 = each context's own form, which
+    may be one CTA per instance; resident CTAs per SM the kernel is compiled for (1 or
+    2, 0 = 2), persistent clusters (0 = all that fit)."""
     _fields_ = [("sub_cluster", ctypes.c_int32 * 3), ("min_blocks", ctypes.c_int32), ("clusters", ctypes.c_int32)]
 
     @classmethod
