@@ -15,6 +15,7 @@
 #include "qhd_device.cuh"
 #include "qhd_group.h"
 #include "qhd_kernels.h"
+#include "qhd_launch.cuh"
 #include "qhd_trace.h"
 #include "qhd_sched.cuh"
 #include "qhd_spectrum.h"
@@ -635,6 +636,14 @@ PrepArgs prep_args(const qhd_ctx *c, int64_t nsteps, double dt) {
     return pa;
 }
 
+// The step tables release the passes of a step at their start, where one badly placed
+// pass costs nothing, and whole-run kernels, which keep their place for a chunk, at
+// their end; of those only a lone instance's at the start (qhd_launch.cuh).
+bool prep_early(const qhd_ctx *c, int64_t cnt) {
+    const bool whole = c->ndim == 1 || c->plane_mode == 2;
+    return !whole || (c->ndim == 2 && c->batch == 1 && cnt > OVERLAP_STEPS);
+}
+
 // Arguments of a chunk's launches of the 2-D whole-run engine: of its one-CTA part
 // (the first c->solo instances) and of the rest, on clusters (the same arrays from its
 // first instance on).
@@ -749,7 +758,7 @@ qhd_status qhd_evolve(qhd_ctx *c, double T, double dt) {
         pa.cnt = cnt;
         {
             TimedScope ts(c, QHD_KCLASS_PREP, true);
-            QHD_LAUNCH(c, launch_prep(pa, c->stream));
+            QHD_LAUNCH(c, launch_prep(pa, prep_early(c, cnt), c->stream));
         }
         if (ndim == 1) {
             OneDArgs o{};
@@ -1162,7 +1171,7 @@ cudaError_t ctx_whole_enqueue(const qhd_ctx *c, int64_t nsteps, double dt, cudaS
     const int64_t ch = c->kt_shared ? c->L.chunk_shared : c->L.chunk;
     for (pa.j0 = 0; pa.j0 < nsteps; pa.j0 += ch) {
         pa.cnt = std::min(ch, nsteps - pa.j0);
-        cudaError_t e = launch_prep(pa, s);
+        cudaError_t e = launch_prep(pa, prep_early(c, pa.cnt), s);
         ++*launches;
         for (const bool solo : {true, false}) {
             const PlaneArgs w = whole_args(c, pa, pa.j0 + pa.cnt == nsteps, solo);

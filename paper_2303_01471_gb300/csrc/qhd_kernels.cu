@@ -55,7 +55,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 4) k_row(RowArgs a) {
     using Sync = std::conditional_t<(T > 32), BlockSync, WarpSync>;
     extern __shared__ __align__(16) float4 smem4[];
     float4 *ptab = smem4;
-    grid_release_upto(TINY_GRID);
+    if (!(a.mode & MODE_FWD)) grid_release();
+    else grid_release_upto(TINY_GRID);
     load_phase_tab(ptab, a.ptab);
     __syncthreads();
     const int line = threadIdx.x / T, t = threadIdx.x % T;
@@ -329,14 +330,15 @@ __global__ void k_prep(PrepArgs a) {
     // the schedules and the potential's scale were loaded under a synchronisation,
     // the tables are read by the passes before: compute first, wait, then write
     const bool row = jl < a.cnt && b < a.kt_batch;
-    const bool one = row && (int)threadIdx.x < a.ksum;
-    const float4 first = one ? prep_kinetic_entry(a, threadIdx.x, s_k, s_fd) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int i0 = (int)(blockIdx.z * blockDim.x + threadIdx.x), stride = (int)(gridDim.z * blockDim.x);
+    const bool one = row && i0 < a.ksum;
+    const float4 first = one ? prep_kinetic_entry(a, i0, s_k, s_fd) : make_float4(0.f, 0.f, 0.f, 0.f);
     grid_wait();
-    if (threadIdx.x == 0) a.pot[jl * a.batch + b] = pot;
+    if (threadIdx.x == 0 && blockIdx.z == 0) a.pot[jl * a.batch + b] = pot;
     if (one) {
         float4 *out = a.kt + (jl * a.kt_batch + b) * a.ksum;
-        out[threadIdx.x] = first;
-        for (int i = threadIdx.x + blockDim.x; i < a.ksum; i += blockDim.x) out[i] = prep_kinetic_entry(a, i, s_k, s_fd);
+        out[i0] = first;
+        for (int i = i0 + stride; i < a.ksum; i += stride) out[i] = prep_kinetic_entry(a, i, s_k, s_fd);
     }
     if (!EARLY) grid_release();
 }
@@ -597,10 +599,13 @@ cudaError_t launch_row(int n, const RowArgs &a, cudaStream_t s) { QHD_DISPATCH_N
 cudaError_t launch_axis(int n, const AxisArgs &a, cudaStream_t s) { QHD_DISPATCH_N(n, axis_impl, a, s) }
 cudaError_t launch_oned(int n, const OneDArgs &a, cudaStream_t s) { QHD_DISPATCH_N(n, oned_impl, a, s) }
 
-cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
-    dim3 grid((unsigned)(a.cnt + 1), (unsigned)a.batch);
-    return launch_overlapped(true, a.batch == 1 && a.cnt > OVERLAP_STEPS ? k_prep<true> : k_prep<false>, grid, dim3(256), 0, s,
-                             a);
+cudaError_t launch_prep(const PrepArgs &a, bool early, cudaStream_t s) {
+    // FP64 bounds a row's entries (1.7 FMA per clock and SM): short chunks of few
+    // instances share each row among blocks (1024^2 x 2, 8 evolutions of 3 steps: 985 us
+    // with a block per row, 832 so)
+    const int64_t split = (a.ksum + 255) / 256;
+    dim3 grid((unsigned)(a.cnt + 1), (unsigned)a.batch, (a.cnt + 1) * a.batch * split <= 152 * 8 ? (unsigned)split : 1u);
+    return launch_overlapped(true, early ? k_prep<true> : k_prep<false>, grid, dim3(256), 0, s, a);
 }
 
 cudaError_t load_prep() {

@@ -145,7 +145,7 @@ struct ObsArgs {
 cudaError_t launch_row(int n, const RowArgs &a, cudaStream_t s);
 cudaError_t launch_axis(int n, const AxisArgs &a, cudaStream_t s);
 cudaError_t launch_oned(int n, const OneDArgs &a, cudaStream_t s);
-cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s);
+cudaError_t launch_prep(const PrepArgs &a, bool early, cudaStream_t s);  // early: releases the next kernel at its start
 // Loads launch_prep's kernels (a first launch inside a stream capture must not).
 cudaError_t load_prep();
 cudaError_t launch_uniform(float2 *psi, int64_t count, float value, cudaStream_t s);

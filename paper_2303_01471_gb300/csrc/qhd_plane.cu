@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(Solo<N1, N2>::THREADS, solo_min_blocks<Solo<N1
     const uint32_t *fq = a.fq + plane * (int64_t)N1 * N2;
     const float4 *tw_row = a.tw_row + P::V * TW2_TABLE * N2;
     const bool inv = a.mode & MODE_INV, fwd = a.mode & MODE_FWD;
+    if (!fwd) grid_release();
     load_phase_tab(ptab, a.ptab);
     grid_wait();
     const uint64_t coef = a.pot[plane >> a.log_planes];
@@ -77,6 +78,7 @@ __global__ void __launch_bounds__(Plane2<N1, N2, C, 1>::THREADS, plane2_min_bloc
     // row blocks) go to L2 now, during the tile load and the inverse transform (20 steps of
     // 256^3: 4871 us without, 4822 with)
     static_assert(P::R % C == 0, "whole rows per CTA");
+    if (!fwd) grid_release();
     if (tid < C) {
         const uint32_t *rows = fq + (int64_t)(P::R * tid + rank * (P::R / C)) * N2;
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(rows), "r"(P::R / C * N2 * 4) : "memory");
