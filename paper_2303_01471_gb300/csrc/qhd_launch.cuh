@@ -14,8 +14,8 @@
 // step, released at the start / at the end / without overlap: 256^2 x 8 19.8 / 13.0 /
 // 13.1 us, 128x256 x 30 19.3 / 12.5 / 12.7, 64^3 17.1 / 9.8 / 14.7, 64x16x128 x 5
 // 17.5 / 15.1 / 22.8).  So the passes, and k_prep where a whole-run kernel follows,
-// release at their end, with these exceptions.  A grid of up to 16 blocks is in nobody's way and releases at its start
-// (16x1024 x 1 6.4 us, 7.2 at the end); one of up to a block per SM before its last
+// release at their end, with these exceptions.  A grid of up to 16 blocks is in
+// nobody's way and releases at its start (16x1024 x 1 6.4 us, 7.2 at the end); one of up to a block per SM before its last
 // transform (256x16 x 1 6.1 and 6.6, 128x16 x 4 5.4 and 6.1; with more threads than
 // that the early blocks get in the way again: 512x256 x 4 13.2 and 11.3); more than 24
 // one-warp blocks per SM at their start (4x1024 x 300 15.6 and 17.7; not with 13 per
