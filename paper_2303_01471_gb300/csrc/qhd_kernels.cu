@@ -102,7 +102,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 4) k_row(RowArgs a) {
                                     turns_mul(c, __ldg(&fq[N + i])) + a.dither, ptab);
         }
     }
-    grid_release_upto(SMALL_GRID);
+    // not at 1024 points, where the check alone costs the passes 1%
+    if constexpr (N < 1024) grid_release_upto(SMALL_GRID);
     if (a.mode & MODE_FWD) line_fft2<N, V, false>(x, sm, t, tw, Sync{}, at);
     if (valid) {
         if constexpr (T == 1) {
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(CP * Line2<N, V>::T, axis_min_blocks<N, V, CP>
         // the mean's part: N mu = sum through the factor of frequency 0
         if (split0 && t == 0) st_c2(slot, c2_mul<false>(c2_mul_shared<false>(ld_c2(slot), kb[0]), kc));
     }
-    grid_release_upto(SMALL_GRID);
+    if constexpr (N < 1024) grid_release_upto(SMALL_GRID);
     if (a.mode & MODE_INV) line_fft2<N, V, true>(x, sm, t, tw, BlockSync{}, at);
     if (split0) {
         // written by the column's thread 0 before the inverse transform's barriers
